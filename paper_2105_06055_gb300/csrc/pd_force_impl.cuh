@@ -9,6 +9,7 @@
 // State-based model with 3 kappa != 5 mu (Eq. 92, 95-97) adds the dilatation
 // round trip between the two halves (see force_state below).
 #pragma once
+#include "pd_horizon.cuh"
 #include "pd_ops.cuh"
 
 namespace pd {
@@ -248,12 +249,9 @@ pd_status weight_gfield(pd_plan *p, const T *s, const uint8_t *lam, T *G, cudaSt
         return PD_ERR_ARG;
     }
     if (s)
-        k_gfield<T, T, T><<<nblk_f(p->N, 128), 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi, s, G,
-                                                           p->N);
+        PD_TRY((launch_gfield<T, T>(p, s, G, nullptr, st)));
     else
-        k_gfield<T, uint8_t, T><<<nblk_f(p->N, 128), 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi,
-                                                                 lam, G, p->N);
-    PD_LAUNCH_CHECK();
+        PD_TRY((launch_gfield<T, uint8_t>(p, lam, G, nullptr, st)));
     p->launches++;
     return PD_OK;
 }

@@ -11,6 +11,7 @@
 #include <map>
 #include <mutex>
 
+#include "pd_horizon.cuh"
 #include "pd_plan.cuh"
 
 namespace pd {
@@ -911,7 +912,7 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
     PD_CUDA_TRY(cudaMemcpyAsync(d_g, hz.g.data(), sizeof(double) * 3 * hz.cnt, cudaMemcpyHostToDevice, st));
     PD_CUDA_TRY(cudaMemcpyAsync(d_w2, hz.w2.data(), sizeof(double) * hz.cnt, cudaMemcpyHostToDevice, st));
     PD_CUDA_TRY(cudaMemcpyAsync(d_cs, hz.cs.data(), sizeof(double) * hz.cnt, cudaMemcpyHostToDevice, st));
-    HorizonDev hd{d_off, d_c, d_g, d_w2, p->nonlinear ? d_cs : nullptr, hz.cnt};
+    HorizonDev hd{d_off, d_c, d_g, d_w2, p->nonlinear ? d_cs : nullptr, hz.cnt, {r[0], r[1], r[2]}};
     p->hdev = hd;
 
     // reduction scratch; the last 64 bytes hold the device status word
@@ -991,9 +992,7 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
     // boundary fields
     PD_TRY(dalloc(p, &p->G64, sizeof(double) * nc * N));
     PD_TRY(dalloc(p, &p->G32, sizeof(float) * nc * N));
-    k_gfield<double, double, double><<<nblk(N, 128), 128, 0, st>>>(n1, n2, n3, hd, nc, p->chi, (const double *)nullptr,
-                                                                 p->G64, N);
-    PD_LAUNCH_CHECK();
+    PD_TRY((launch_gfield<double, double>(p, nullptr, p->G64, nullptr, st)));
     k_convert<float><<<nblk(nc * N), 256, 0, st>>>(p->G64, p->G32, nc * N);
     PD_LAUNCH_CHECK();
     {

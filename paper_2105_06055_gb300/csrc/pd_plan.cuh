@@ -54,35 +54,9 @@ struct HorizonDev {
     const double *w2; // cnt: omega |xi|^2 dV
     const double *cs; // cnt: c(xi) dV = alpha / |xi|^3 dV (nonlinear bond model), or null
     int cnt;
+    int r[3];         // reach along each axis, in cells (the offsets' order is symmetric: bond
+                      // cnt - 1 - c is opposite to bond c)
 };
-
-// Boundary field of a node weight v = chi s (Eq. 100 with the difference kernel):
-//   G_c(x) = Σ_H C_c(xi) dV (v(x+xi) - v(x)),  G = 0 where chi = 0.
-// For v = chi this is -(Σ_H C dV (1 - chi(x+xi))): zero in the delta-interior.
-template <typename T, typename V, typename Acc>
-__global__ void k_gfield(int n1, int n2, int n3, HorizonDev hz, int ncomp, const uint8_t *chi,
-                         const V *s, T *G, int64_t N)
-{
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    int i1, i2, i3;
-    node_coords(p, n1, n2, i1, i2, i3);
-    Acc acc[6] = {0, 0, 0, 0, 0, 0};
-    if (chi[p]) {
-        const Acc vp = s ? (Acc)s[p] : Acc(1);
-        for (int c = 0; c < hz.cnt; ++c) {
-            const int a = (i1 + hz.off[3 * c]) & (n1 - 1);
-            const int b = (i2 + hz.off[3 * c + 1]) & (n2 - 1);
-            const int e = (i3 + hz.off[3 * c + 2]) & (n3 - 1);
-            const int64_t q = ((int64_t)e * n2 + b) * n1 + a;
-            const Acc vq = chi[q] ? (s ? (Acc)s[q] : Acc(1)) : Acc(0);
-            const Acc dv = vq - vp;
-            if (dv != Acc(0))
-                for (int k = 0; k < ncomp; ++k) acc[k] += (Acc)hz.c[k * hz.cnt + c] * dv;
-        }
-    }
-    for (int k = 0; k < ncomp; ++k) G[k * N + p] = (T)acc[k];
-}
 
 // Kernel-spectrum lookup from a tile's shared-memory slice (component stride cs)
 template <typename T>

@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "pd_horizon.cuh"
 #include "pd_ops.cuh"
 #include "pd_plan.cuh"
 
@@ -70,34 +71,6 @@ __global__ void k_kick(T *v, const T *L, const T *b, const uint8_t *co, int64_t 
 {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
         v[q] = co[q] ? v[q] + hdt_rho * (L[q] + b[q]) : T(0);
-}
-
-// G^lam_c(x) = Σ_H C_c dV (v(x+xi) - v(x)), v = chi lam; skipped unless the
-// change flag is set by this step's kick-drift (k_clear_changed resets it).
-template <typename T>
-__global__ void k_gfield_lam(int n1, int n2, int n3, HorizonDev hz, int ncomp, const uint8_t *chi,
-                             const uint8_t *lam, T *G, int64_t N, VerletCounters *cnt, int force)
-{
-    if (!force && !cnt->changed) return;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < N) {
-        int i1, i2, i3;
-        node_coords(p, n1, n2, i1, i2, i3);
-        T acc[6] = {0, 0, 0, 0, 0, 0};
-        if (chi[p]) {
-            const T vp = lam[p] ? T(1) : T(0);
-            for (int c = 0; c < hz.cnt; ++c) {
-                const int a = (i1 + hz.off[3 * c]) & (n1 - 1);
-                const int bb = (i2 + hz.off[3 * c + 1]) & (n2 - 1);
-                const int e = (i3 + hz.off[3 * c + 2]) & (n3 - 1);
-                const int64_t q = ((int64_t)e * n2 + bb) * n1 + a;
-                const T dv = ((chi[q] && lam[q]) ? T(1) : T(0)) - vp;
-                if (dv != T(0))
-                    for (int k = 0; k < ncomp; ++k) acc[k] += (T)hz.c[k * hz.cnt + c] * dv;
-            }
-        }
-        for (int k = 0; k < ncomp; ++k) G[k * N + p] = acc[k];
-    }
 }
 
 __global__ void k_clear_changed(VerletCounters *cnt) { cnt->changed = 0; }
@@ -152,10 +125,89 @@ __global__ void k_energy_direct(int n1, int n2, int n3, HorizonDev hz, double dx
     }
 }
 
+// The same sum on shared-memory tiles (pd_horizon.cuh): the weight mask and u
+// of a tile with its halo are loaded once, the bond table is a few vectors per
+// bond, shared by the thread's kNodes nodes.
+template <typename T, int D>
+__global__ void __launch_bounds__(kHzX *kHzY)
+    k_energy_tile(HzTile t, HorizonDev hz, double dx1, double dx2, double dx3, const uint8_t *__restrict__ chi,
+                  const uint8_t *__restrict__ lam, const T *__restrict__ u, T *__restrict__ W, int64_t N)
+{
+    constexpr int NC = Sym<D>::n;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    T *bond = reinterpret_cast<T *>(sm_raw);             // [cnt][4]: xi, c / |xi|^2
+    int *off = reinterpret_cast<int *>(bond + 4 * hz.cnt);
+    T *tu = reinterpret_cast<T *>(off + ((hz.cnt + 3) & ~3));  // [D][tile], 0 where the weight is 0
+    const int tile = t.p * t.rows * t.nz;
+    uint8_t *tm = reinterpret_cast<uint8_t *>(tu + (size_t)D * tile);  // weight mask
+    const int tid = threadIdx.y * kHzX + threadIdx.x;
+    for (int c = tid; c < hz.cnt; c += kHzX * kHzY) {
+        const double x[3] = {hz.off[3 * c] * dx1, hz.off[3 * c + 1] * dx2, hz.off[3 * c + 2] * dx3};
+        double tr = 0.0, r2 = 0.0;
+        for (int k = 0; k < NC; ++k)
+            if (Sym<D>::i(k) == Sym<D>::j(k)) tr += hz.c[k * hz.cnt + c];
+        for (int j = 0; j < D; ++j) r2 += x[j] * x[j];
+        for (int j = 0; j < 3; ++j) bond[4 * c + j] = j < D ? (T)x[j] : T(0);
+        bond[4 * c + 3] = (T)(tr / r2);
+        off[c] = (hz.off[3 * c + 2] * t.rows + hz.off[3 * c + 1]) * t.p + hz.off[3 * c];
+    }
+    hz_fill(t, [&](int e, int64_t q) {
+        const bool in = chi[q] && lam[q];
+        tm[e] = in ? 1 : 0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) tu[j * tile + e] = in ? u[j * N + q] : T(0);
+    });
+    __syncthreads();
+    const int e0 = hz_elem0(t);
+    T up[kNodes][D], acc[kNodes];
+#pragma unroll
+    for (int m = 0; m < kNodes; ++m) {
+        acc[m] = T(0);
+#pragma unroll
+        for (int j = 0; j < D; ++j) up[m][j] = tu[j * tile + e0 + m * t.step];
+    }
+#pragma unroll 2
+    for (int c = 0; c < hz.cnt; ++c) {
+        const int d = e0 + off[c];
+        T x[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[j] = bond[4 * c + j];
+        const T w = bond[4 * c + 3];
+#pragma unroll
+        for (int m = 0; m < kNodes; ++m) {
+            const int e = d + m * t.step;
+            T s = T(0);
+#pragma unroll
+            for (int j = 0; j < D; ++j) s += x[j] * (tu[j * tile + e] - up[m][j]);
+            const T next = acc[m] + w * s * s;
+            acc[m] = tm[e] ? next : acc[m];
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < kNodes; ++m) {
+        int64_t p;
+        if (hz_node(t, m, p)) W[p] = tm[e0 + m * t.step] ? T(0.5) * acc[m] : T(0);
+    }
+}
+
 template <typename T>
 pd_status energy_direct(pd_plan *p, const T *u, const uint8_t *lam, T *W, cudaStream_t st)
 {
     const int cnt = p->hdev.cnt;
+    {
+        const HzTile t = hz_tile(p->dim, p->n1, p->n2, p->n3, p->hdev);
+        const size_t ts = (size_t)4 * cnt * sizeof(T) + (size_t)((cnt + 3) & ~3) * sizeof(int) +
+                          (size_t)t.p * t.rows * t.nz * (p->dim * sizeof(T) + 1);
+        if (ts <= kHzSmem) {
+            const auto kern = p->dim == 3 ? k_energy_tile<T, 3> : k_energy_tile<T, 2>;
+            PD_TRY(set_smem_attr((const void *)kern, ts));
+            kern<<<hz_grid(t), dim3(kHzX, kHzY), ts, st>>>(t, p->hdev, p->prob.dx[0], p->prob.dx[1], p->prob.dx[2],
+                                                           p->chi, lam, u, W, p->N);
+            PD_LAUNCH_CHECK();
+            p->launches++;
+            return PD_OK;
+        }
+    }
     const size_t smem = (size_t)(1 + p->dim) * cnt * sizeof(T) + (size_t)3 * cnt * sizeof(int);
     const double *dx = p->prob.dx;
     const unsigned ng = (unsigned)std::min<int64_t>(8 * p->nsm, (p->N + 255) / 256);
@@ -197,10 +249,8 @@ pd_status verlet_impl(pd_plan *p, T *u, T *v, uint8_t *lam, const T *b, const T 
     const int breaking = (lam && p->wc > 0) ? 1 : 0;
     VerletCounters *cnt = reinterpret_cast<VerletCounters *>(p->red + kRedVerlet);
     PD_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(VerletCounters), st));
-    const unsigned nbl = (unsigned)((N + 127) / 128);
     if (lam) {
-        k_gfield_lam<T><<<nbl, 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi, lam, G, N, cnt, 1);
-        PD_LAUNCH_CHECK();
+        PD_TRY((launch_gfield<T, uint8_t>(p, lam, G, nullptr, st)));
         p->launches++;
     }
     PD_TRY(step_force<T>(p, u, lam, G, L, W, breaking, st));
@@ -214,7 +264,8 @@ pd_status verlet_impl(pd_plan *p, T *u, T *v, uint8_t *lam, const T *b, const T 
         PD_LAUNCH_CHECK();
         p->launches++;
         if (breaking) {
-            k_gfield_lam<T><<<nbl, 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi, lam, G, N, cnt, 0);
+            // G^lam, skipped unless this step's kick-drift flagged a change
+            PD_TRY((launch_gfield<T, uint8_t>(p, lam, G, &cnt->changed, st)));
             k_clear_changed<<<1, 1, 0, st>>>(cnt);
             PD_LAUNCH_CHECK();
             p->launches += 2;

@@ -30,6 +30,7 @@
 #include <cmath>
 #include <vector>
 
+#include "pd_horizon.cuh"
 #include "pd_ops.cuh"
 #include "pd_plan.cuh"
 
@@ -68,32 +69,6 @@ __global__ void k_adj_weight(const T *s, const uint8_t *lam, T *s_eff, int64_t N
 {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
         s_eff[p] = lam[p] ? s[p] : T(0);
-}
-
-// boundary field of the weight v = chi s_eff (as k_gfield), skipped unless flagged
-template <typename T>
-__global__ void k_adj_gfield(int n1, int n2, int n3, HorizonDev hz, int ncomp, const uint8_t *chi, const T *s,
-                             T *G, int64_t N, const AdjCounters *cnt)
-{
-    if (!cnt->changed) return;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    int i1, i2, i3;
-    node_coords(p, n1, n2, i1, i2, i3);
-    T acc[6] = {0, 0, 0, 0, 0, 0};
-    if (chi[p]) {
-        const T vp = s[p];
-        for (int c = 0; c < hz.cnt; ++c) {
-            const int a = (i1 + hz.off[3 * c]) & (n1 - 1);
-            const int b = (i2 + hz.off[3 * c + 1]) & (n2 - 1);
-            const int e = (i3 + hz.off[3 * c + 2]) & (n3 - 1);
-            const int64_t q = ((int64_t)e * n2 + b) * n1 + a;
-            const T dv = (chi[q] ? s[q] : T(0)) - vp;
-            if (dv != T(0))
-                for (int k = 0; k < ncomp; ++k) acc[k] += (T)hz.c[k * hz.cnt + c] * dv;
-        }
-    }
-    for (int k = 0; k < ncomp; ++k) G[k * N + p] = acc[k];
 }
 
 __global__ void k_adj_flag(AdjCounters *cnt, int v) { cnt->changed = v; }
@@ -237,7 +212,7 @@ struct AdjRun {
     AdjCounters *cnt;
     T h, dt;
     int breaking;
-    unsigned ng, ngv, nbl;
+    unsigned ng, ngv;
 
     T *ck_u(int k) const { return (T *)(w + lay.ck_u) + (size_t)k * p->dim * p->N; }
     T *ck_v(int k) const { return (T *)(w + lay.ck_v) + (size_t)k * p->dim * p->N; }
@@ -251,7 +226,7 @@ struct AdjRun {
     {
         k_adj_weight<T><<<ng, 256, 0, st>>>(s, lam, seff, p->N);
         if (force_g) k_adj_flag<<<1, 1, 0, st>>>(cnt, 1);
-        k_adj_gfield<T><<<nbl, 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi, seff, G, p->N, cnt);
+        PD_TRY((launch_gfield<T, T>(p, seff, G, &cnt->changed, st)));
         k_adj_flag<<<1, 1, 0, st>>>(cnt, 0);
         PD_LAUNCH_CHECK();
         p->launches += force_g ? 4 : 3;
@@ -312,7 +287,6 @@ pd_status loss_grad_impl(pd_plan *p, const T *c_rel, const uint8_t *lam0, const 
     const int64_t N = p->N, dN = (int64_t)p->dim * N;
     R.ng = (unsigned)std::min<int64_t>(4 * p->nsm, (N + 255) / 256);
     R.ngv = (unsigned)std::min<int64_t>(4 * p->nsm, (dN + 255) / 256);
-    R.nbl = (unsigned)((N + 127) / 128);
     const size_t vb = sizeof(T) * (size_t)dN;
 
     PD_CUDA_TRY(cudaMemsetAsync(R.cnt, 0, sizeof(AdjCounters), st));
@@ -390,8 +364,7 @@ pd_status loss_grad_impl(pd_plan *p, const T *c_rel, const uint8_t *lam0, const 
                 PD_TRY(R.copy(R.lam, R.sg_lam(n - k0), (size_t)N));
                 k_adj_weight<T><<<R.ng, 256, 0, st>>>(R.s, R.lam, R.seff, N);
                 k_adj_flag<<<1, 1, 0, st>>>(R.cnt, 1);
-                k_adj_gfield<T><<<R.nbl, 128, 0, st>>>(p->n1, p->n2, p->n3, p->hdev, p->ncomp, p->chi, R.seff,
-                                                       R.G, N, R.cnt);
+                PD_TRY((launch_gfield<T, T>(p, R.seff, R.G, &R.cnt->changed, st)));
                 PD_LAUNCH_CHECK();
                 p->launches += 3;
             }
