@@ -51,11 +51,14 @@ struct AffineView {
 
 // Block partial sums of the fit: Σ chi u_j (D values) and Σ chi e_k u_j
 // (D^2 values, index D + D j + k), in compensated FP32 (FP64 for FP64 fields).
-template <typename T, int D>
+// NV = D: the first D sums only (the body mean). One block_sums exchange for
+// all sums: FP32 pairs are merged per warp and only one lane per warp and sum
+// touches FP64 (a separate FP64 block reduction per sum kept the FP64 pipe busy
+// for 60 us of a 64^3 evaluation).
+template <typename T, int D, int NV = D + D * D>
 __global__ void __launch_bounds__(256) k_aff_sums(const T *u, const uint8_t *chi, int lg1, int lg2, int c0, int c1,
                                                   int c2, int64_t N, double *red)
 {
-    constexpr int NV = D + D * D;
     DSum acc[NV];
     pdl_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
@@ -66,16 +69,36 @@ __global__ void __launch_bounds__(256) k_aff_sums(const T *u, const uint8_t *chi
         for (int j = 0; j < D; ++j) {
             const T uj = u[j * N + p];
             acc[j].add(uj);
+            if constexpr (NV > D) {
 #pragma unroll
-            for (int k = 0; k < D; ++k) acc[D + D * j + k].add(e[k] * uj);
+                for (int k = 0; k < D; ++k) acc[D + D * j + k].add(e[k] * uj);
+            }
         }
     }
     pdl_trigger();
+    const DSum *a[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const double t = block_sum_d(acc[v].value());
-        if (threadIdx.x == 0) red[kRedPart + (int64_t)blockIdx.x * NV + v] = t;
+    for (int v = 0; v < NV; ++v) a[v] = &acc[v];
+    double t[NV];
+    block_sums<NV>(a, t);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) red[kRedPart + (int64_t)blockIdx.x * NV + v] = t[v];
     }
+}
+
+// sums[v] = Σ over nblk block partials of value v, one warp per value (256 threads)
+template <int NV>
+__device__ __forceinline__ void aff_total(const double *red, int nblk, double *sums)
+{
+    const int lane = threadIdx.x & 31;
+    for (int v = threadIdx.x >> 5; v < NV; v += 8) {
+        double s = 0.0;
+        for (int b = lane; b < nblk; b += 32) s += red[kRedPart + (int64_t)b * NV + v];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) sums[v] = s;
+    }
+    __syncthreads();
 }
 
 struct AffFitArgs {
@@ -91,13 +114,7 @@ __global__ void __launch_bounds__(256) k_aff_fit(const double *red, AffFitArgs a
     constexpr int NV = D + D * D;
     __shared__ double sums[NV];
     pdl_wait();
-    for (int v = 0; v < NV; ++v) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < a.nblk; b += blockDim.x) s += red[kRedPart + (int64_t)b * NV + v];
-        s = block_sum_d(s);
-        if (threadIdx.x == 0) sums[v] = s;
-        __syncthreads();
-    }
+    aff_total<NV>(red, a.nblk, sums);
     pdl_trigger();
     if (threadIdx.x != 0) return;
     constexpr int M = D + 1;

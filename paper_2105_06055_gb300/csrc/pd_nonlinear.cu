@@ -44,21 +44,14 @@ struct NL {
     static constexpr int P = 0, A = D, B = D + D * D, CC = D + D * D + NS;
 };
 
-// the body mean of u (from the affine-fit block sums) as the coefficient t of
+// the body mean of u (from the block sums) as the coefficient t of
 // an AffineView with B = 0 (one block)
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_nl_mean(const double *red, int nblk, double inv_count, T *coef)
 {
-    constexpr int NV = D + D * D;
     __shared__ double sums[D];
     pdl_wait();
-    for (int v = 0; v < D; ++v) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += red[kRedPart + (int64_t)b * NV + v];
-        s = block_sum_d(s);
-        if (threadIdx.x == 0) sums[v] = s;
-        __syncthreads();
-    }
+    aff_total<D>(red, nblk, sums);
     pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < 9; ++k) coef[k] = T(0);
@@ -288,7 +281,7 @@ pd_status force_nl_dim(pd_plan *p, const T *u, T *L, cudaStream_t st)
     {
         constexpr int kBlocks = 296;
         const int lg1 = ilog2(p->n1), lg2 = ilog2(p->n2);
-        PD_TRY(launch_k(p->pdl != 0, k_aff_sums<T, D>, dim3(kBlocks), dim3(256), 0, st, u,
+        PD_TRY(launch_k(p->pdl != 0, k_aff_sums<T, D, D>, dim3(kBlocks), dim3(256), 0, st, u,
                         (const uint8_t *)p->chi, lg1, lg2, p->aff_c[0], p->aff_c[1], p->aff_c[2], p->N, p->red));
         PD_TRY(launch_k(p->pdl != 0, k_nl_mean<T, D>, dim3(1), dim3(256), 0, st, (const double *)p->red, kBlocks,
                         p->body_count > 0 ? 1.0 / p->body_count : 0.0, coef));
