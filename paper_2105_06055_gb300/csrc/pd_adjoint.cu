@@ -20,12 +20,35 @@ pd_status weight_gfield(pd_plan *p, const T *s, const uint8_t *lam, T *G, cudaSt
 
 namespace {
 
+// Two consecutive values of a caller's field, which may start on any element:
+// one vector access when it starts on a pair's boundary.
+template <typename T>
+__device__ __forceinline__ void load_two(bool pairs, const T *p, T &a, T &b)
+{
+    if (pairs) {
+        load_pair(p, a, b);
+    } else {
+        a = p[0];
+        b = p[1];
+    }
+}
+template <typename T>
+__device__ __forceinline__ void store_two(bool pairs, T *p, T a, T b)
+{
+    if (pairs) {
+        store2(p, a, b);
+    } else {
+        p[0] = a;
+        p[1] = b;
+    }
+}
+
 template <typename T, int D>
 struct ProAdj {
     static constexpr int NC = Sym<D>::n;
-    static constexpr int kFin = 0, kFout = 2 * D + NC, kNF = 0, kNB = 0, kStage = 0;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = 0, kFout = 2 * D + NC, kNB = 0, kDim = D;
     const T *u, *pv, *s;
+    bool pairs;  // they start on pair boundaries
     const uint8_t *chi;
     int64_t N;
     int n1;
@@ -33,27 +56,33 @@ struct ProAdj {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int) const { return nullptr; }
     __device__ cx<T> *spec_out(int f) const { return spec + f * fstride; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return nullptr; }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
     __device__ void block_done(DSum &) const {}
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *, const T *, T *o0,
-                                          T *o1) const
+    struct Nd {
+        T ua[D], ub[D], pa[D], pb[D], sa, sb;
+        uchar2 in;
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        node(c.row0 + rl, i1, o0);
-        node(c.row0 + rl, i1 + 1, o1);
-    }
-    __device__ __forceinline__ void node(int64_t row, int i1, T *out) const
-    {
-        const int64_t q = row * n1 + i1;
-        T v = chi[q] ? T(1) : T(0);
-        if (s) v *= s[q];
-        T uu[D], pp[D];
+        nd.in = *reinterpret_cast<const uchar2 *>(chi + p0 + o);
+        nd.sa = nd.sb = T(1);
+        if (s) load_two(pairs, s + p0 + o, nd.sa, nd.sb);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            uu[j] = u[j * N + q];
-            pp[j] = pv[j * N + q];
+            load_two(pairs, u + (j * N + p0) + o, nd.ua[j], nd.ub[j]);
+            load_two(pairs, pv + (j * N + p0) + o, nd.pa[j], nd.pb[j]);
+        }
+    }
+    __device__ __forceinline__ void node2(const RowCtx &, int, Nd &nd, const T *, const T *, T *o0, T *o1,
+                                          DSum &) const
+    {
+        node(nd.in.x ? nd.sa : T(0) * nd.sa, nd.ua, nd.pa, o0);
+        node(nd.in.y ? nd.sb : T(0) * nd.sb, nd.ub, nd.pb, o1);
+    }
+    __device__ __forceinline__ void node(T v, const T *uu, const T *pp, T *out) const
+    {
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
             out[j] = v * uu[j];
             out[D + j] = v * pp[j];
         }
@@ -68,18 +97,15 @@ struct ProAdj {
 template <typename T, int D>
 struct CombAdj {
     static constexpr int NC = Sym<D>::n;
-    static constexpr int kFin = 2 * D + NC, kFout = 2 * D + 1, kMode = 2, kPre = 0, kTab = NC;
-    static constexpr bool kStoreIn = false;
+    static constexpr int kFin = 2 * D + NC, kFout = 2 * D + 1, kTab = NC, kDim = D;
     Model<T> m;
-    int obase;  // first output slot (out of place in 3D)
     __device__ int slot_in(int f) const { return f; }
-    __device__ int slot_out(int f) const { return obase + f; }
-    __device__ int slot_aux(int) const { return 0; }
+    __device__ int slot_out(int f) const { return f; }
     __device__ const T *table(int c) const { return m.mhat + c * m.fold_sz; }
-    __device__ __forceinline__ void combine(const T *t, int cs, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
+    __device__ __forceinline__ void combine(const T *t, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
     {
         T M[9];
-        load_mhat_s(D, t, cs, fy, fz, M);
+        load_mhat_s(D, t, fy, fz, M);
         mat_vec<T, D>(M, in, out);
         mat_vec<T, D>(M, in + D, out + D);
         cx<T> acc = mk(T(0), T(0));
@@ -96,64 +122,64 @@ struct CombAdj {
 template <typename T, int D>
 struct EpiAdj {
     static constexpr int NC = Sym<D>::n;
-    static constexpr int kFin = 2 * D + 1, kFout = 0, kNF = 0, kNB = 0, kStage = 0;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = 2 * D + 1, kFout = 0, kNB = 0, kDim = D;
     const T *u, *pv, *s, *G;
     const uint8_t *chi;
     T *gu, *gs;
+    bool pairs;  // u, pv, s, gu and gs start on pair boundaries
     int64_t N;
     int n1;
     const cx<T> *spec;
     int64_t fstride;
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return nullptr; }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
     __device__ void block_done(DSum &) const {}
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *,
-                                          T *) const
+    struct Nd {
+        T ua[D], ub[D], pa[D], pb[D], ga[NC], gb[NC], sa, sb;
+        uchar2 in;
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        node(c.row0 + rl, i1, in0);
-        node(c.row0 + rl, i1 + 1, in1);
-    }
-    __device__ __forceinline__ void node(int64_t row, int i1, const T *in) const
-    {
-        const int64_t q = row * n1 + i1;
-        const bool inb = chi[q] != 0;
-        T v = inb ? T(1) : T(0);
-        if (s) v *= s[q];
-        T uu[D], pp[D], Gu[D], Gp[D];
+        nd.in = *reinterpret_cast<const uchar2 *>(chi + p0 + o);
+        nd.sa = nd.sb = T(1);
+        if (s) load_two(pairs, s + p0 + o, nd.sa, nd.sb);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            uu[j] = u[j * N + q];
-            pp[j] = pv[j * N + q];
-            Gu[j] = Gp[j] = T(0);
+            load_two(pairs, u + (j * N + p0) + o, nd.ua[j], nd.ub[j]);
+            load_two(pairs, pv + (j * N + p0) + o, nd.pa[j], nd.pb[j]);
         }
-        if (inb) {
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const int a = Sym<D>::i(c), b = Sym<D>::j(c);
-                const T g = G[c * N + q];
-                Gu[a] += g * uu[b];
-                Gp[a] += g * pp[b];
-                if (a != b) {
-                    Gu[b] += g * uu[a];
-                    Gp[b] += g * pp[a];
-                }
-            }
-        }
+        for (int k = 0; k < NC; ++k) load_pair(G + (k * N + p0) + o, nd.ga[k], nd.gb[k]);
+    }
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *in0, const T *in1, T *, T *,
+                                          DSum &) const
+    {
+        T xa[D], xb[D], ya, yb;
+        node(nd.in.x != 0, nd.in.x ? nd.sa : T(0) * nd.sa, nd.ua, nd.pa, nd.ga, in0, xa, ya);
+        node(nd.in.y != 0, nd.in.y ? nd.sb : T(0) * nd.sb, nd.ub, nd.pb, nd.gb, in1, xb, yb);
         if (gu) {
 #pragma unroll
-            for (int i = 0; i < D; ++i) gu[i * N + q] = v * (in[D + i] - Gp[i]);
+            for (int i = 0; i < D; ++i) store_two(pairs, gu + (i * N + c.p0) + o, xa[i], xb[i]);
         }
-        if (gs) {
-            T acc = -in[2 * D];
+        if (gs) store_two(pairs, gs + c.p0 + o, ya, yb);
+    }
+    __device__ __forceinline__ void node(bool inb, T v, const T *uu, const T *pp, const T *g, const T *in, T *x,
+                                         T &y) const
+    {
+        T Gu[D], Gp[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) acc += pp[i] * in[i] - pp[i] * Gu[i] + uu[i] * in[D + i];
-            gs[q] = inb ? acc : T(0);
+        for (int j = 0; j < D; ++j) Gu[j] = Gp[j] = T(0);
+        if (inb) {
+            sym_apply<T, D>(g, uu, Gu);
+            sym_apply<T, D>(g, pp, Gp);
         }
+#pragma unroll
+        for (int i = 0; i < D; ++i) x[i] = v * (in[D + i] - Gp[i]);
+        T acc = -in[2 * D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) acc += pp[i] * in[i] - pp[i] * Gu[i] + uu[i] * in[D + i];
+        y = inb ? acc : T(0);
     }
 };
 
@@ -164,14 +190,15 @@ pd_status adjoint_pipeline(pd_plan *p, const T *u, const T *s, const T *pv, cons
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     constexpr int FI = 2 * D + Sym<D>::n, FO = 2 * D + 1;
-    ProAdj<T, D> pro{u, pv, s, p->chi, p->N, p->n1, spec, fs};
+    const uintptr_t any = (uintptr_t)u | (uintptr_t)pv | (uintptr_t)s | (uintptr_t)gu | (uintptr_t)gs;
+    const bool pairs = any % (2 * sizeof(T)) == 0;
+    ProAdj<T, D> pro{u, pv, s, pairs, p->chi, p->N, p->n1, spec, fs};
     PD_TRY(launch_rows<T>(p, pro, st));
-    if (D == 3) PD_TRY((col_pass<T, FI>(p, 0, false, st)));
-    const int ob = D == 3 ? FI : 0;
-    CombAdj<T, D> cmb{model_view<T>(p), ob};
-    PD_TRY(launch_cols<T>(p, cmb, D == 3 ? 2 : 1, true, FI, st));
-    if (D == 3) PD_TRY((col_pass<T, FO>(p, ob, true, st)));
-    EpiAdj<T, D> epi{u, pv, s, G, p->chi, gu, gs, p->N, p->n1, spec + ob * fs, fs};
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, FI, false, st));
+    CombAdj<T, D> cmb{model_view<T>(p)};
+    PD_TRY(launch_comb<T>(p, cmb, st));
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, FO, true, st));
+    EpiAdj<T, D> epi{u, pv, s, G, p->chi, gu, gs, pairs, p->N, p->n1, spec, fs};
     PD_TRY(launch_rows<T>(p, epi, st));
     return PD_OK;
 }

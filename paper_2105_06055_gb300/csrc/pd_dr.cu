@@ -250,8 +250,7 @@ __device__ __forceinline__ void dr_accumulate(DrAcc &acc, T Fn, T r, T ee)
 // rows, forward: v^{n+1/2}, e^{n+1} from c^n, F^n; transform chi v
 template <typename T, int D>
 struct ProDR {
-    static constexpr int kFin = 0, kFout = D, kNF = 0, kNB = 1, kStage = 0;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = 0, kFout = D, kNB = 1, kDim = D;
     T *e, *v;
     const T *F;
     const uint8_t *chi;
@@ -262,48 +261,50 @@ struct ProDR {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int) const { return nullptr; }
     __device__ cx<T> *spec_out(int f) const { return spec + f * fstride; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return chi; }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *, const T *, T *o0,
-                                          T *o1) const
+    struct Nd {
+        typename vec2<T>::type ev[D], vv[D], fv[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
+    {
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            nd.ev[j] = load2(e + (j * N + p0) + o);
+            nd.vv[j] = load2(v + (j * N + p0) + o);
+            nd.fv[j] = load2(F + (j * N + p0) + o);
+        }
+    }
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *, const T *, T *o0, T *o1,
+                                          DSum &) const
     {
         const T cd = (T)scal[R_C], rinv = (T)scal[R_RHOINV];
         const T a = (T(2) - cd) / (T(2) + cd), bf = T(2) * rinv / (T(2) + cd);
-        const T m0 = c.b(0, rl, i1) ? T(1) : T(0), m1 = c.b(0, rl, i1 + 1) ? T(1) : T(0);
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        typename vec2<T>::type ev[D], vv[D], fv[D];
+        T m0, m1;
+        chi_pair(c, o, m0, m1);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            ev[j] = load2(e + j * N + p);
-            vv[j] = load2(v + j * N + p);
-            fv[j] = load2(F + j * N + p);
-        }
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            const T va = a * vv[j].x + bf * fv[j].x, vb = a * vv[j].y + bf * fv[j].y;
-            const T ea = ev[j].x + va, eb = ev[j].y + vb;
-            store2(v + j * N + p, va, vb);
-            store2(e + j * N + p, ea, eb);
+            const T va = a * nd.vv[j].x + bf * nd.fv[j].x, vb = a * nd.vv[j].y + bf * nd.fv[j].y;
+            const T ea = nd.ev[j].x + va, eb = nd.ev[j].y + vb;
+            store2(v + (j * N + c.p0) + o, va, vb);
+            store2(e + (j * N + c.p0) + o, ea, eb);
             o0[j] = m0 * va;
             o1[j] = m1 * vb;
         }
     }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
     __device__ void block_done(DSum &) const {}
 };
 
-// rows, inverse: L(v) = chi y - G v staged, F^{n+1} = F^n + chi_O L(v), partials
+// rows, inverse: L(v) = chi y - G v, F^{n+1} = F^n + chi_O L(v), partials
 template <typename T, int D>
 struct EpiDR {
-    static constexpr int kFin = D, kFout = 0, kStage = D, kNF = 0, kNB = 1 + D;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = D, kFout = 0, kNB = 1, kDim = D;
+    static constexpr bool kReduce = true, kEntries = true;
     using Acc = DrAcc;
     const T *e, *v, *rhs;
     T *F;
-    const uint8_t *chi, *co;
+    const uint8_t *bits;  // bit 0 chi, bit 1 + i chi_Omega of component i
     const GEntry<T> *gent;
-    const int *gidx;
+    const int *goff;
     double *red;
     int64_t N;
     int n1;
@@ -311,23 +312,12 @@ struct EpiDR {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
-    __device__ const T *nf_src(int) const { return nullptr; }
-    __device__ const uint8_t *nb_src(int k) const { return k == 0 ? chi : co + (k - 1) * N; }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *o0,
-                                          T *o1) const
-    {
-        const T m0 = c.b(0, rl, i1) ? T(1) : T(0), m1 = c.b(0, rl, i1 + 1) ? T(1) : T(0);
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            o0[i] = m0 * in0[i];
-            o1[i] = m1 * in1[i];
-        }
-    }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    // L -= G v at a boundary node (entry k of the list)
-    __device__ __forceinline__ void fix(int64_t p, int k, T *s) const
+    __device__ const uint8_t *nb_src(int) const { return bits; }
+    __device__ __forceinline__ const int *rows_off() const { return goff; }
+    __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {
         const GEntry<T> g = gent[k];
+        p = g.p;
         T vv[D], Gv[D];
 #pragma unroll
         for (int q = 0; q < D; ++q) {
@@ -336,35 +326,32 @@ struct EpiDR {
         }
         sym_apply<T, D>(g.g, vv, Gv);
 #pragma unroll
-        for (int i = 0; i < D; ++i) s[i] -= Gv[i];
+        for (int i = 0; i < D; ++i) s[i] = -Gv[i];
     }
-    __device__ __forceinline__ void emit(const RowCtx<T> &c, int rl, int i1, const T *s0, const T *s1,
-                                         DrAcc &acc) const
-    {
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        const int2 gi = *reinterpret_cast<const int2 *>(gidx + p);
-        T a[D], b[D];
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            a[i] = s0[i];
-            b[i] = s1[i];
-        }
-        if (gi.x >= 0) fix(p, gi.x, a);
-        if (gi.y >= 0) fix(p + 1, gi.y, b);
+    struct Nd {
         typename vec2<T>::type ev[D], rv[D], fv[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
+    {
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            ev[i] = load2(e + i * N + p);
-            rv[i] = load2(rhs + i * N + p);
-            fv[i] = load2(F + i * N + p);
+            nd.ev[i] = load2(e + (i * N + p0) + o);
+            nd.rv[i] = load2(rhs + (i * N + p0) + o);
+            nd.fv[i] = load2(F + (i * N + p0) + o);
         }
+    }
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *in0, const T *in1, T *, T *,
+                                          DrAcc &acc) const
+    {
+        const uchar2 m = c.b2(0, o);
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            const T fa = c.b(1 + i, rl, i1) ? fv[i].x + a[i] : T(0);
-            const T fb = c.b(1 + i, rl, i1 + 1) ? fv[i].y + b[i] : T(0);
-            store2(F + i * N + p, fa, fb);
-            dr_accumulate<T>(acc, fa, rv[i].x, ev[i].x);
-            dr_accumulate<T>(acc, fb, rv[i].y, ev[i].y);
+            const T a = (m.x & 1) ? in0[i] : T(0), b = (m.y & 1) ? in1[i] : T(0);
+            const T fa = ((m.x >> (1 + i)) & 1) ? nd.fv[i].x + a : T(0);
+            const T fb = ((m.y >> (1 + i)) & 1) ? nd.fv[i].y + b : T(0);
+            store2(F + (i * N + c.p0) + o, fa, fb);
+            dr_accumulate<T>(acc, fa, nd.rv[i].x, nd.ev[i].x);
+            dr_accumulate<T>(acc, fb, nd.rv[i].y, nd.ev[i].y);
         }
     }
     __device__ void block_done(DrAcc &acc) const { write_partial3(red, acc); }
@@ -454,12 +441,11 @@ struct DrSpec {
         const Model<T> m = model_view<T>(p);
         ProDR<T, D> pro{e, v, F, p->chi, p->red + kRedScal, p->N, p->n1, spec, fs};
         PD_TRY(launch_rows<T>(p, pro, st));
-        if (D == 3) PD_TRY((col_pass<T, D>(p, 0, false, st)));
-        const int ob = D == 3 ? D : 0;
-        CombForce<T, D, false> cmb{m, ob};
-        PD_TRY(launch_cols<T>(p, cmb, D == 3 ? 2 : 1, true, D, st));
-        if (D == 3) PD_TRY((col_pass<T, D>(p, ob, true, st)));
-        EpiDR<T, D> epi{e, v, rhs, F, p->chi, p->chi_om, m.gent, p->gidx, p->red, p->N, p->n1, spec + ob * fs, fs};
+        if (D == 3) PD_TRY(col_pass<T>(p, 0, D, false, st));
+            CombForce<T, D, false> cmb{m};
+        PD_TRY(launch_comb<T>(p, cmb, st));
+        if (D == 3) PD_TRY(col_pass<T>(p, 0, D, true, st));
+        EpiDR<T, D> epi{e, v, rhs, F, p->mbits, m.gent, p->goff, p->red, p->N, p->n1, spec, fs};
         unsigned gepi = 0;
         PD_TRY(launch_rows<T>(p, epi, st, &gepi));
         if (gepi > (unsigned)kDrPart) {

@@ -16,8 +16,6 @@ namespace pd {
 
 static inline unsigned nblk_f(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
 
-// SPARSE: the epilogue takes the plan's boundary-node list of G (weight chi_B);
-// otherwise the dense G passed in (weight chi_B, chi_B s or chi_B lam).
 // Fit of the affine split (pd_affine.cuh): block sums over the body, then the
 // exact-form coefficients in the plan's coefficient buffer.
 template <typename T, int D>
@@ -38,33 +36,33 @@ pd_status affine_fit(pd_plan *p, const T *u, cudaStream_t st, AffineView<T> *vie
     return PD_OK;
 }
 
-template <typename T, int D, bool ENERGY, int WM, bool SPARSE = (WM == W_NONE), bool AFF = false>
+// Weight chi_B (s = lam = null) or chi_B s or chi_B lam. G null: the epilogue
+// takes the plan's boundary-node list (weight chi_B only), else the dense G of
+// the weight. aff: transform u - a, a the affine fit (list only, no energy).
+template <typename T, int D, bool ENERGY>
 pd_status force_bond_pipeline(pd_plan *p, const T *u, const T *s, const uint8_t *lam, const T *G, T *L, T *W,
-                              cudaStream_t st)
+                              cudaStream_t st, bool aff = false)
 {
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     constexpr int FI = D + (ENERGY ? Sym<D>::n : 0), FO = D + (ENERGY ? 1 : 0);
     AffineView<T> av{};
-    if constexpr (AFF) PD_TRY((affine_fit<T, D>(p, u, st, &av)));
-    ProForce<T, D, ENERGY, WM, AFF> pro{u, s, lam, p->chi, p->N, spec, fs, av};
+    if (aff) PD_TRY((affine_fit<T, D>(p, u, st, &av)));
+    const NodeWeight<T> w{s, lam};
+    ProForce<T, D, ENERGY> pro{u, w, p->chi, p->N, p->n1, spec, fs, av};
     PD_TRY(launch_rows<T>(p, pro, st));
-    if (D == 3) PD_TRY((col_pass<T, FI>(p, 0, false, st)));
-    const int ob = D == 3 ? FI : 0;
-    CombForce<T, D, ENERGY> cmb{model_view<T>(p), ob};
-    PD_TRY(launch_cols<T>(p, cmb, D == 3 ? 2 : 1, true, FI, st));
-    if (D == 3) PD_TRY((col_pass<T, FO>(p, ob, true, st)));
-    if constexpr (SPARSE) {
-        static_assert(WM == W_NONE, "the boundary-node list is for the plan weight chi_B");
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, FI, false, st));
+    CombForce<T, D, ENERGY> cmb{model_view<T>(p)};
+    PD_TRY(launch_comb<T>(p, cmb, st));
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, FO, true, st));
+    if (!G) {
         const Model<T> m = model_view<T>(p);
-        EpiForceSparse<T, D, ENERGY, AFF> epi{u, p->chi, m.gent, p->gidx, L, W, p->N, p->n1, spec + ob * fs, fs,
-                                              av, reinterpret_cast<const T *>(p->aff_tab)};
-        PD_TRY(launch_rows<T>(p, epi, st));
-    } else {
-        EpiForceDense<T, D, ENERGY, WM> epi{u, s, lam, p->chi, G, L, W, p->N, p->n1, spec + ob * fs, fs};
-        PD_TRY(launch_rows<T>(p, epi, st));
+        EpiForceSparse<T, D, ENERGY> epi{u, p->chi, m.gent, p->goff, L, W, p->N, p->n1, spec, fs, av,
+                                         reinterpret_cast<const T *>(p->aff_tab)};
+        return launch_rows<T>(p, epi, st);
     }
-    return PD_OK;
+    EpiForceDense<T, D, ENERGY> epi{u, w, p->chi, G, L, W, p->N, p->n1, spec, fs};
+    return launch_rows<T>(p, epi, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -79,23 +77,21 @@ pd_status force_bond_pipeline(pd_plan *p, const T *u, const T *s, const uint8_t 
 // ghat_i = dV gamma_i / N.
 // ---------------------------------------------------------------------------
 
-// Slots: 0-2 chi u_j (x1, x2 transformed), 3 S, 4 theta, 5-7 fully transformed
-// chi u_j, 0-2 again for the outputs (every 3D last-axis pass writes slots it
-// does not read).
-// last axis, first combine: transform chi u_j (kept in slots 5-7), S = Σ -i ghat_i X_i
+// Slots: 0-2 chi u_j (x1, x2 transformed), 3 S, 4 theta; 0-2 again for the
+// outputs. The second combine transforms chi u_j along x3 once more: cheaper
+// than writing three transformed spectra and reading them back.
+// last axis, first combine: S = Σ -i ghat_i X_i
 template <typename T>
 struct CombTheta {
-    static constexpr int kFin = 3, kFout = 1, kMode = 2, kPre = 0, kTab = 3;
-    static constexpr bool kStoreIn = true;
+    static constexpr int kFin = 3, kFout = 1, kTab = 3, kDim = 3;
     Model<T> m;
     __device__ int slot_in(int f) const { return f; }
-    __device__ int slot_aux(int f) const { return 5 + f; }
     __device__ int slot_out(int) const { return 3; }
     __device__ const T *table(int c) const { return m.ghat + c * m.fold_sz; }
-    __device__ __forceinline__ void combine(const T *t, int cs, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
+    __device__ __forceinline__ void combine(const T *t, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
     {
         T g[3];
-        load_ghat_s(t, cs, fy, fz, g);
+        load_ghat_s(t, fy, fz, g);
         cx<T> acc = mk(T(0), T(0));
 #pragma unroll
         for (int i = 0; i < 3; ++i) acc = acc + scale(in[i], g[i]);
@@ -106,8 +102,7 @@ struct CombTheta {
 // rows: inverse of S, theta at the nodes, forward transform of theta
 template <typename T>
 struct RowTheta {
-    static constexpr int kFin = 1, kFout = 1, kNF = 0, kNB = 0, kStage = 0;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = 1, kFout = 1, kNB = 0, kDim = 3;
     Model<T> m;
     const T *u;
     T *theta;
@@ -115,48 +110,51 @@ struct RowTheta {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int) const { return spec + 3 * fstride; }
     __device__ cx<T> *spec_out(int) const { return spec + 4 * fstride; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return nullptr; }
-    __device__ __forceinline__ T node1(int64_t p, T in) const
+    struct Nd {
+        T ma, mb, ga[3], gb[3], ua[3], ub[3];
+        uchar2 in;
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        T th = T(0);
-        if (m.chi[p]) {
-            T qu = T(0);
+        load_pair(m.m3inv + p0 + o, nd.ma, nd.mb);
+        nd.in = *reinterpret_cast<const uchar2 *>(m.chi + p0 + o);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) qu += m.qt[i * m.N + p] * u[i * m.N + p];
-            th = -m.m3inv[p] * (in + qu);
+        for (int i = 0; i < 3; ++i) {
+            load_pair(m.qt + (i * m.N + p0) + o, nd.ga[i], nd.gb[i]);
+            load_pair(u + (i * m.N + p0) + o, nd.ua[i], nd.ub[i]);
         }
-        return th;
     }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *o0,
-                                          T *o1) const
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *in0, const T *in1, T *o0,
+                                          T *o1, DSum &) const
     {
-        const int64_t p = (c.row0 + rl) * m.n1 + i1;
-        const T t0 = node1(p, in0[0]), t1 = node1(p + 1, in1[0]);
-        store2(theta + p, t0, t1);
+        T qa = T(0), qb = T(0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            qa += nd.ga[i] * nd.ua[i];
+            qb += nd.gb[i] * nd.ub[i];
+        }
+        const T t0 = nd.in.x ? -nd.ma * (in0[0] + qa) : T(0), t1 = nd.in.y ? -nd.mb * (in1[0] + qb) : T(0);
+        store2(theta + c.p0 + o, t0, t1);
         o0[0] = t0;
         o1[0] = t1;
     }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
     __device__ void block_done(DSum &) const {}
 };
 
 // last axis, second combine: Y_i = M^_ij X_j + i ka ghat_i Theta
 template <typename T>
 struct CombState {
-    static constexpr int kFin = 4, kFout = 3, kMode = 2, kPre = 3, kTab = 9;
-    static constexpr bool kStoreIn = false;
+    static constexpr int kFin = 4, kFout = 3, kTab = 9, kDim = 3;
     Model<T> m;
-    __device__ int slot_in(int f) const { return f < 3 ? 5 + f : 4; }
+    __device__ int slot_in(int f) const { return f < 3 ? f : 4; }
     __device__ int slot_out(int f) const { return f; }
-    __device__ int slot_aux(int) const { return 0; }
     __device__ const T *table(int c) const { return c < 6 ? m.mhat + c * m.fold_sz : m.ghat + (c - 6) * m.fold_sz; }
-    __device__ __forceinline__ void combine(const T *t, int cs, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
+    __device__ __forceinline__ void combine(const T *t, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
     {
         T M[9], g[3];
-        load_mhat_s(3, t, cs, fy, fz, M);
-        load_ghat_s(t + 6 * cs, cs, fy, fz, g);
+        load_mhat_s(3, t, fy, fz, M);
+        load_ghat_s(t + 6, fy, fz, g);
         mat_vec<T, 3>(M, in, out);
         const cx<T> it = mul_i(in[3]);
 #pragma unroll
@@ -164,12 +162,12 @@ struct CombState {
     }
 };
 
-// rows: inverse of Y, L = chi y staged, boundary fix-up
+// rows: inverse of Y, L = chi y, boundary nodes:
 //   L_i -= G_ij u_j - ka theta q_i   (q_i and G vanish off the boundary list)
 template <typename T>
 struct EpiState {
-    static constexpr int kFin = 3, kFout = 0, kNF = 0, kNB = 1, kStage = 3;
-    static constexpr bool kSparse = true;
+    static constexpr int kFin = 3, kFout = 0, kNB = 1, kDim = 3;
+    static constexpr bool kEntries = true;
     Model<T> m;
     const T *u;
     const T *theta;
@@ -178,41 +176,29 @@ struct EpiState {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return m.chi; }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *o0,
-                                          T *o1) const
+    __device__ __forceinline__ const int *rows_off() const { return m.goff; }
+    __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {
-        const T v0 = c.b(0, rl, i1) ? T(1) : T(0), v1 = c.b(0, rl, i1 + 1) ? T(1) : T(0);
+        const GEntry<T> e = m.gent[k];
+        p = e.p;
+        T uu[3], Gu[3] = {T(0), T(0), T(0)};
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            o0[i] = v0 * in0[i];
-            o1[i] = v1 * in1[i];
-        }
+        for (int j = 0; j < 3; ++j) uu[j] = u[j * m.N + p];
+        sym_apply<T, 3>(e.g, uu, Gu);
+        const T th = theta[p];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) s[i] = m.ka * th * m.qt[i * m.N + p] - Gu[i];
     }
-    __device__ void sparse(const RowCtx<T> &c, int tid, int nthreads) const
+    struct Nd {
+    };
+    __device__ __forceinline__ void load(Nd &, int64_t, int) const {}
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &, const T *in0, const T *in1, T *, T *,
+                                          DSum &) const
     {
-        const int64_t N = m.N;
-        const int k0 = m.goff[c.row0], k1 = m.goff[c.row0 + c.rows];
-        for (int k = k0 + tid; k < k1; k += nthreads) {
-            const GEntry<T> e = m.gent[k];
-            const int64_t p = e.p;
-            const int rl = (int)(p / m.n1 - c.row0), i1 = (int)(p % m.n1);
-            T uu[3], Gu[3] = {T(0), T(0), T(0)};
+        const uchar2 b = c.b2(0, o);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) uu[j] = u[j * N + p];
-            sym_apply<T, 3>(e.g, uu, Gu);
-            const T th = theta[p];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) c.stage(i, rl, i1) -= Gu[i] - m.ka * th * m.qt[i * N + p];
-        }
-    }
-    __device__ __forceinline__ void emit(const RowCtx<T> &c, int rl, int i1, const T *s0, const T *s1,
-                                         DSum &) const
-    {
-        const int64_t p = (c.row0 + rl) * m.n1 + i1;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) store2(L + i * m.N + p, s0[i], s1[i]);
+        for (int i = 0; i < 3; ++i) store2(L + (i * m.N + c.p0) + o, b.x ? in0[i] : T(0), b.y ? in1[i] : T(0));
     }
     __device__ void block_done(DSum &) const {}
 };
@@ -223,18 +209,18 @@ pd_status force_state_pipeline(pd_plan *p, const T *u, T *L, T *theta, cudaStrea
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     const Model<T> m = model_view<T>(p);
-    ProForce<T, 3, false, W_NONE> pro{u, nullptr, nullptr, p->chi, p->N, spec, fs};
+    ProForce<T, 3, false> pro{u, NodeWeight<T>{nullptr, nullptr}, p->chi, p->N, p->n1, spec, fs, AffineView<T>{}};
     PD_TRY(launch_rows<T>(p, pro, st));
-    PD_TRY((col_pass<T, 3>(p, 0, false, st)));
+    PD_TRY(col_pass<T>(p, 0, 3, false, st));
     CombTheta<T> c1{m};
-    PD_TRY(launch_cols<T>(p, c1, 2, true, 3, st));
-    PD_TRY((col_pass<T, 1>(p, 3, true, st)));
+    PD_TRY(launch_comb<T>(p, c1, st));
+    PD_TRY(col_pass<T>(p, 3, 1, true, st));
     RowTheta<T> rt{m, u, theta, spec, fs};
     PD_TRY(launch_rows<T>(p, rt, st));
-    PD_TRY((col_pass<T, 1>(p, 4, false, st)));
+    PD_TRY(col_pass<T>(p, 4, 1, false, st));
     CombState<T> c2{m};
-    PD_TRY(launch_cols<T>(p, c2, 2, true, 4, st));
-    PD_TRY((col_pass<T, 3>(p, 0, true, st)));
+    PD_TRY(launch_comb<T>(p, c2, st));
+    PD_TRY(col_pass<T>(p, 0, 3, true, st));
     EpiState<T> epi{m, u, theta, L, spec, fs};
     PD_TRY(launch_rows<T>(p, epi, st));
     return PD_OK;
@@ -266,19 +252,13 @@ pd_status force_any(pd_plan *p, const T *u, const T *s, const uint8_t *lam, cons
         set_error("force: s and lambda together are not supported");
         return PD_ERR_ARG;
     }
-#define PD_FORCE_CASE(D, E)                                                                         \
-    do {                                                                                            \
-        if (s) return force_bond_pipeline<T, D, E, W_S>(p, u, s, lam, G, L, W, st);                 \
-        if (lam) return force_bond_pipeline<T, D, E, W_LAM>(p, u, s, lam, G, L, W, st);             \
-        return force_bond_pipeline<T, D, E, W_NONE>(p, u, s, lam, G, L, W, st);                     \
-    } while (0)
+    const T *g = s || lam ? G : nullptr;  // weight chi_B: the plan's list
     if (p->dim == 2) {
-        if (W) PD_FORCE_CASE(2, true);
-        PD_FORCE_CASE(2, false);
+        if (W) return force_bond_pipeline<T, 2, true>(p, u, s, lam, g, L, W, st);
+        return force_bond_pipeline<T, 2, false>(p, u, s, lam, g, L, W, st);
     }
-    if (W) PD_FORCE_CASE(3, true);
-    PD_FORCE_CASE(3, false);
-#undef PD_FORCE_CASE
+    if (W) return force_bond_pipeline<T, 3, true>(p, u, s, lam, g, L, W, st);
+    return force_bond_pipeline<T, 3, false>(p, u, s, lam, g, L, W, st);
 }
 
 template <typename T>
@@ -320,9 +300,29 @@ pd_status force_public(pd_plan *p, const T *u, const T *s, T *L, T *W, cudaStrea
 {
     const bool aff = p->affine_split && !p->state_based && !s && !W && sizeof(T) == (p->prob.fp64 ? 8 : 4);
     if (!aff) return force_plain<T>(p, u, s, L, W, st);
-    if (p->dim == 2) return force_bond_pipeline<T, 2, false, W_NONE, true, true>(p, u, s, nullptr, nullptr, L, W, st);
-    return force_bond_pipeline<T, 3, false, W_NONE, true, true>(p, u, s, nullptr, nullptr, L, W, st);
+    if (p->dim == 2) return force_bond_pipeline<T, 2, false>(p, u, s, nullptr, nullptr, L, W, st, true);
+    return force_bond_pipeline<T, 3, false>(p, u, s, nullptr, nullptr, L, W, st, true);
 }
+
+// Instantiated once per precision, in pd_force_f32.cu and pd_force_f64.cu.
+#define PD_FORCE_INSTANCES(EXTERN, T)                                                                             \
+    EXTERN template pd_status weight_gfield<T>(pd_plan *, const T *, const uint8_t *, T *, cudaStream_t);          \
+    EXTERN template pd_status force_any<T>(pd_plan *, const T *, const T *, const uint8_t *, const T *, T *, T *,  \
+                                           cudaStream_t);                                                          \
+    EXTERN template pd_status force_plain<T>(pd_plan *, const T *, const T *, T *, T *, cudaStream_t);             \
+    EXTERN template pd_status force_public<T>(pd_plan *, const T *, const T *, T *, T *, cudaStream_t);            \
+    EXTERN template pd_status force_bond_pipeline<T, 2, false>(pd_plan *, const T *, const T *, const uint8_t *,   \
+                                                               const T *, T *, T *, cudaStream_t, bool);           \
+    EXTERN template pd_status launch_comb<T, CombForce<T, 2, false>>(pd_plan *, const CombForce<T, 2, false> &,    \
+                                                                     cudaStream_t);                                \
+    EXTERN template pd_status launch_comb<T, CombForce<T, 3, false>>(pd_plan *, const CombForce<T, 3, false> &,    \
+                                                                     cudaStream_t);
+#ifndef PD_FORCE_UNIT_F32
+PD_FORCE_INSTANCES(extern, float)
+#endif
+#ifndef PD_FORCE_UNIT_F64
+PD_FORCE_INSTANCES(extern, double)
+#endif
 
 }  // namespace pd
 

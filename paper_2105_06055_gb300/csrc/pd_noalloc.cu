@@ -116,13 +116,16 @@ __global__ void k_na_fold(int n1, int n2, int h, const int *off, const double *c
     for (int q = 0; q < 3; ++q) mhat[q * fold_sz + t] = (float)(acc[q] * invN);
 }
 
-__global__ void k_na_twiddle(cx<float> *tw, int L)
+// the twiddle tables of every length up to 2^lgmax and stage radix (pd_cols.cuh)
+__global__ void k_na_twiddle(cx<float> *tw, int lgmax)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= L) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= tw_entries(lgmax)) return;
+    const int k = 31 - __clz(t / kTwRadices + 1), o = t - tw_base(k, 0), r = o >> k, i = o & ((1 << k) - 1);
+    const int e = r ? (i >> r) * (i & ((1 << r) - 1)) : i;
     double s, c;
-    sincospi(2.0 * (double)k / (double)L, &s, &c);
-    tw[k] = mk((float)c, (float)-s);
+    sincospi(2.0 * (double)(e & ((1 << k) - 1)) / (double)(1 << k), &s, &c);
+    tw[t] = mk((float)c, (float)-s);
 }
 
 // The body must stay delta away from the box faces and chi must be 0/1.
@@ -199,12 +202,11 @@ extern "C" pd_status pd_force2d_noalloc(const pd_problem *pr, const uint8_t *chi
     const int h = n1 / 2;
     const int64_t fold = (int64_t)(h + 1) * (n2 / 2 + 1);
     const int lgl = ilog2(std::max(n1, n2));
-    const int L2 = 1 << lgl;
     // carve the scratch array
     const size_t b_spec = up256(sizeof(float) * 2 * (size_t)N);  // two packed spectra (2D pass is in place)
     const size_t b_G = up256(sizeof(float) * 3 * (size_t)N);
     const size_t b_mh = up256(sizeof(float) * 3 * (size_t)fold);
-    const size_t b_tw = up256(sizeof(cx<float>) * (size_t)L2);
+    const size_t b_tw = up256(sizeof(cx<float>) * (size_t)tw_entries(lgl));
     const size_t b_off = up256(sizeof(int) * 3 * (size_t)cnt);
     const size_t b_c = up256(sizeof(double) * 3 * (size_t)cnt);
     const size_t b_flag = 256;
@@ -240,7 +242,7 @@ extern "C" pd_status pd_force2d_noalloc(const pd_problem *pr, const uint8_t *chi
     const double alpha = 9.0 * pr->E / (M_PI * pr->delta * pr->delta * pr->delta);
     k_na_horizon<<<1, 32, 0, st>>>(r1, r2, pr->dx[0], pr->dx[1], pr->delta, alpha, dV, off, cc, cnt);
     k_na_fold<<<(unsigned)((fold + 127) / 128), 128, 0, st>>>(n1, n2, h, off, cc, cnt, 1.0 / (double)N, mh, fold);
-    k_na_twiddle<<<(L2 + 255) / 256, 256, 0, st>>>(tw, L2);
+    k_na_twiddle<<<(tw_entries(lgl) + 255) / 256, 256, 0, st>>>(tw, lgl);
     PD_LAUNCH_CHECK();
     HorizonDev hd{off, cc, nullptr, nullptr, nullptr, cnt, {r1, r2, 0}};
     k_gfield<float, double, double><<<(unsigned)((N + 127) / 128), 128, 0, st>>>(n1, n2, 1, hd, 3, chi_B,
@@ -281,7 +283,7 @@ extern "C" pd_status pd_force2d_noalloc(const pd_problem *pr, const uint8_t *chi
         PD_CUDA_TRY(cudaGetDevice(&dev));
         PD_CUDA_TRY(cudaDeviceGetAttribute(&p.nsm, cudaDevAttrMultiProcessorCount, dev));
     }
-    const pd_status s = force_bond_pipeline<float, 2, false, W_NONE, false>(&p, u, nullptr, nullptr, G, L, nullptr, st);
+    const pd_status s = force_bond_pipeline<float, 2, false>(&p, u, nullptr, nullptr, G, L, nullptr, st);
     // the stack plan owns nothing: detach its views before it goes out of scope
     p.chi = nullptr;
     p.mhat32 = nullptr;

@@ -63,27 +63,23 @@ __global__ void __launch_bounds__(256) k_nl_mean(const double *red, int nblk, do
 template <typename T, int D>
 struct ProNL {
     using K = NL<D>;
-    static constexpr int kFin = 0, kFout = K::FWD, kNF = D, kNB = 1, kStage = 0;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = 0, kFout = K::FWD, kNB = 1, kDim = D;
     const T *u;
     const uint8_t *chi;
     int64_t N;
+    int n1;
     cx<T> *spec;
     int64_t fstride;
     AffineView<T> mean;
     __device__ const cx<T> *spec_in(int) const { return nullptr; }
     __device__ cx<T> *spec_out(int f) const { return spec + f * fstride; }
-    __device__ const T *nf_src(int k) const { return u + k * N; }
     __device__ const uint8_t *nb_src(int) const { return chi; }
-    __device__ __forceinline__ void node1(const RowCtx<T> &c, int rl, int i1, T *out) const
+    __device__ __forceinline__ void node1(T v, const T *m, const T *un, T *out) const
     {
-        const T v = c.b(0, rl, i1) ? T(1) : T(0);
-        T m[D], uu[D];
-        mean.at(i1, c.row0 + rl, D, m);
-        T s2 = T(0);
+        T uu[D], s2 = T(0);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            uu[j] = c.f(j, rl, i1) - m[j];
+            uu[j] = un[j] - m[j];
             s2 += uu[j] * uu[j];
         }
 #pragma unroll
@@ -94,25 +90,35 @@ struct ProNL {
 #pragma unroll
         for (int q = 0; q < K::NS; ++q) out[K::Y + q] = v * uu[Sym<D>::i(q)] * uu[Sym<D>::j(q)];
     }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *, const T *, T *o0,
-                                          T *o1) const
+    struct Nd {
+        T a[D], b[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        node1(c, rl, i1, o0);
-        node1(c, rl, i1 + 1, o1);
+#pragma unroll
+        for (int j = 0; j < D; ++j) load_pair(u + (j * N + p0) + o, nd.a[j], nd.b[j]);
     }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *, const T *, T *o0, T *o1,
+                                          DSum &) const
+    {
+        T va, vb, m[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) m[j] = mean.coef[kAffT + j];
+        chi_pair(c, o, va, vb);
+        node1(va, m, nd.a, o0);
+        node1(vb, m, nd.b, o1);
+    }
     __device__ void block_done(DSum &) const {}
 };
 
-// odd-kernel spectrum g_i from a table slice (component stride cs): the
-// components along folded axes change sign
+// odd-kernel spectrum g_i from a mode's table values: the components along
+// folded axes change sign
 template <typename T, int D>
-__device__ __forceinline__ void load_odd(const T *t, int cs, bool fy, bool fz, T *g)
+__device__ __forceinline__ void load_odd(const T *t, bool fy, bool fz, T *g)
 {
     g[0] = t[0];
-    g[1] = fy ? -t[cs] : t[cs];
-    if (D == 3) g[2] = fz ? -t[2 * cs] : t[2 * cs];
+    g[1] = fy ? -t[1] : t[1];
+    if (D == 3) g[2] = fz ? -t[2] : t[2];
 }
 
 // Spectral combination of the seven (2D) or twelve (3D) forward fields into
@@ -120,24 +126,21 @@ __device__ __forceinline__ void load_odd(const T *t, int cs, bool fy, bool fz, T
 template <typename T, int D>
 struct CombNL {
     using K = NL<D>;
-    static constexpr int kFin = K::FWD, kFout = K::INV, kMode = 2, kPre = 0, kTab = K::NS + 1 + D;
-    static constexpr bool kStoreIn = false;
+    static constexpr int kFin = K::FWD, kFout = K::INV, kTab = K::NS + 1 + D, kDim = D;
     const T *mhat, *chat, *ghat;
     int64_t fold_sz;
-    int obase;  // first output slot (3D: after the inputs, the pass is out of place)
     __device__ int slot_in(int f) const { return f; }
-    __device__ int slot_out(int f) const { return obase + f; }
-    __device__ int slot_aux(int) const { return 0; }
+    __device__ int slot_out(int f) const { return f; }
     __device__ const T *table(int c) const
     {
         return c < K::NS ? mhat + c * fold_sz : (c == K::NS ? chat : ghat + (c - K::NS - 1) * fold_sz);
     }
-    __device__ __forceinline__ void combine(const T *t, int cs, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
+    __device__ __forceinline__ void combine(const T *t, bool fy, bool fz, const cx<T> *in, cx<T> *out) const
     {
         T M[9], g[3];
-        load_mhat_s(D, t, cs, fy, fz, M);
-        const T ch = t[K::NS * cs];
-        load_odd<T, D>(t + (K::NS + 1) * cs, cs, fy, fz, g);
+        load_mhat_s(D, t, fy, fz, M);
+        const T ch = t[K::NS];
+        load_odd<T, D>(t + K::NS + 1, fy, fz, g);
         auto Yf = [&](int i, int j) -> cx<T> {
             const int a = i < j ? i : j, b = i < j ? j : i;
 #pragma unroll
@@ -176,13 +179,14 @@ struct CombNL {
 template <typename T, int D>
 struct EpiNL {
     using K = NL<D>;
-    static constexpr int kFin = K::INV, kFout = 0, kStage = D, kNF = D, kNB = 1;
-    static constexpr bool kSparse = false;
+    static constexpr int kFin = K::INV, kFout = 0, kNB = 1, kDim = D;
+    static constexpr bool kEntries = true;
+    static_assert(K::P == 0, "the boundary entries add to the first D fields");
     const T *u;
     const uint8_t *chi;
     const GEntry<T> *gent;
     const T *nlb;  // [entry][4]: S(a_j, w) (D), S(c, w) - c^(0) w
-    const int *gidx;
+    const int *goff;
     T *L;
     int64_t N;
     int n1;
@@ -191,24 +195,9 @@ struct EpiNL {
     AffineView<T> mean;
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
-    __device__ const T *nf_src(int k) const { return u + k * N; }
     __device__ const uint8_t *nb_src(int) const { return chi; }
-    __device__ __forceinline__ void node_u(const RowCtx<T> &c, int rl, int i1, T *uu, T &s2) const
+    __device__ __forceinline__ void node1(T v, const T *uu, T s2, const T *in, T *o) const
     {
-        T m[D];
-        mean.at(i1, c.row0 + rl, D, m);
-        s2 = T(0);
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            uu[j] = c.f(j, rl, i1) - m[j];
-            s2 += uu[j] * uu[j];
-        }
-    }
-    __device__ __forceinline__ void node1(const RowCtx<T> &c, int rl, int i1, const T *in, T *o) const
-    {
-        const T v = c.b(0, rl, i1) ? T(1) : T(0);
-        T uu[D], s2;
-        node_u(c, rl, i1, uu, s2);
         T trA = T(0), trB = T(0), cu = T(0);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
@@ -227,45 +216,54 @@ struct EpiNL {
             o[i] = v * t;
         }
     }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *o0,
-                                          T *o1) const
-    {
-        node1(c, rl, i1, in0, o0);
-        node1(c, rl, i1 + 1, in1, o1);
-    }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ __forceinline__ void fix(const RowCtx<T> &c, int rl, int i1, int k, T *s) const
+    __device__ __forceinline__ const int *rows_off() const { return goff; }
+    // boundary entry k: its terms go to P_i, which enters L_i as it is
+    __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {
         const GEntry<T> e = gent[k];
         const T *nb = nlb + 4 * (int64_t)k;
-        T uu[D], s2, Gu[D];
-        node_u(c, rl, i1, uu, s2);
-        T sau = T(0);
+        p = e.p;
+        T uu[D], Gu[D], sau = T(0), s2 = T(0);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
+            uu[j] = u[j * N + p] - mean.coef[kAffT + j];
             Gu[j] = T(0);
             sau += nb[j] * uu[j];
+            s2 += uu[j] * uu[j];
         }
         sym_apply<T, D>(e.g, uu, Gu);
         const T sc = nb[3];
 #pragma unroll
-        for (int i = 0; i < D; ++i) s[i] += -Gu[i] + uu[i] * sau + T(0.5) * s2 * (nb[i] - sc * uu[i]);
+        for (int f = D; f < kFin; ++f) s[f] = T(0);
+#pragma unroll
+        for (int i = 0; i < D; ++i) s[K::P + i] = -Gu[i] + uu[i] * sau + T(0.5) * s2 * (nb[i] - sc * uu[i]);
     }
-    __device__ __forceinline__ void emit(const RowCtx<T> &c, int rl, int i1, const T *s0, const T *s1,
-                                         DSum &) const
-    {
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        const int2 gi = *reinterpret_cast<const int2 *>(gidx + p);
+    struct Nd {
         T a[D], b[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
+    {
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-            a[i] = s0[i];
-            b[i] = s1[i];
+        for (int j = 0; j < D; ++j) load_pair(u + (j * N + p0) + o, nd.a[j], nd.b[j]);
+    }
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *in0, const T *in1, T *, T *,
+                                          DSum &) const
+    {
+        T sa = T(0), sb = T(0);
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            const T m = mean.coef[kAffT + j];
+            nd.a[j] -= m;
+            nd.b[j] -= m;
+            sa += nd.a[j] * nd.a[j];
+            sb += nd.b[j] * nd.b[j];
         }
-        if (gi.x >= 0) fix(c, rl, i1, gi.x, a);
-        if (gi.y >= 0) fix(c, rl, i1 + 1, gi.y, b);
+        const uchar2 b = c.b2(0, o);
+        T x[D], y[D];
+        node1(b.x ? T(1) : T(0), nd.a, sa, in0, x);
+        node1(b.y ? T(1) : T(0), nd.b, sb, in1, y);
 #pragma unroll
-        for (int i = 0; i < D; ++i) store2(L + i * N + p, a[i], b[i]);
+        for (int i = 0; i < D; ++i) store2(L + (i * N + c.p0) + o, x[i], y[i]);
     }
     __device__ void block_done(DSum &) const {}
 };
@@ -288,19 +286,18 @@ pd_status force_nl_dim(pd_plan *p, const T *u, T *L, cudaStream_t st)
         p->launches += 2;
     }
     const AffineView<T> mean{coef, p->aff_c[0], p->aff_c[1], p->aff_c[2], ilog2(p->n1), ilog2(p->n2)};
-    ProNL<T, D> pro{u, p->chi, p->N, spec, fs, mean};
+    ProNL<T, D> pro{u, p->chi, p->N, p->n1, spec, fs, mean};
     PD_TRY(launch_rows<T>(p, pro, st));
-    if (D == 3) PD_TRY((col_pass<T, K::FWD>(p, 0, false, st)));
-    const int ob = D == 3 ? K::FWD : 0;
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, K::FWD, false, st));
     const T *mhat = sizeof(T) == 8 ? (const T *)p->mhat64 : (const T *)p->mhat32;
     const T *chat = sizeof(T) == 8 ? (const T *)p->chat64 : (const T *)p->chat32;
     const T *ghat = sizeof(T) == 8 ? (const T *)p->ghat64 : (const T *)p->ghat32;
-    CombNL<T, D> cmb{mhat, chat, ghat, p->fold_sz, ob};
-    PD_TRY(launch_cols<T>(p, cmb, D == 3 ? 2 : 1, true, K::INV, st));
-    if (D == 3) PD_TRY((col_pass<T, K::INV>(p, ob, true, st)));
+    CombNL<T, D> cmb{mhat, chat, ghat, p->fold_sz};
+    PD_TRY(launch_comb<T>(p, cmb, st));
+    if (D == 3) PD_TRY(col_pass<T>(p, 0, K::INV, true, st));
     const Model<T> m = model_view<T>(p);
-    EpiNL<T, D> epi{u, p->chi, m.gent, reinterpret_cast<const T *>(p->nlb), p->gidx, L, p->N, p->n1,
-                    spec + ob * fs, fs, mean};
+    EpiNL<T, D> epi{u, p->chi, m.gent, reinterpret_cast<const T *>(p->nlb), p->goff, L, p->N, p->n1,
+                    spec, fs, mean};
     PD_TRY(launch_rows<T>(p, epi, st));
     return PD_OK;
 }

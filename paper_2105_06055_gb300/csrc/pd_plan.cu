@@ -26,39 +26,6 @@ void set_error(const char *fmt, ...)
     va_end(ap);
 }
 
-pd_status encode_tmap_3d(CUtensorMap *m, void *base, bool fp64, const unsigned long long dims[3],
-                         const unsigned long long strides[2], const unsigned box[3])
-{
-    typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static EncodeFn fn = nullptr;
-    if (!fn) {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000,
-                                                               cudaEnableDefault, &q);
-        if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !f) {
-            set_error("cuTensorMapEncodeTiled is not available from the driver");
-            return PD_ERR_CUDA;
-        }
-        fn = (EncodeFn)f;
-    }
-    const cuuint64_t gd[3] = {dims[0], dims[1], dims[2]};
-    const cuuint64_t gs[2] = {strides[0], strides[1]};
-    const cuuint32_t bx[3] = {box[0], box[1], box[2]};
-    const cuuint32_t es[3] = {1, 1, 1};
-    const CUresult r = fn(m, fp64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, gd, gs,
-                          bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled failed (%d): dims %llu x %llu x %llu, box %u x %u x %u", (int)r, dims[0],
-                  dims[1], dims[2], box[0], box[1], box[2]);
-        return PD_ERR_CUDA;
-    }
-    return PD_OK;
-}
-
 // The dynamic shared-memory limit is a property of the kernel function, shared
 // by every plan and by every kernel node of a captured graph: it only ever
 // grows, so plans of different sizes never lower it under each other.
@@ -337,7 +304,7 @@ __global__ void k_gcount(int n1, int64_t nrows, const uint8_t *chi, const double
 }
 
 __global__ void k_gfill(int n1, int64_t nrows, const uint8_t *chi, const double *G, int nc, int64_t N, const int *off,
-                        GEntry<double> *e64, GEntry<float> *e32, int *gidx)
+                        GEntry<double> *e64, GEntry<float> *e32)
 {
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= nrows) return;
@@ -357,7 +324,6 @@ __global__ void k_gfill(int n1, int64_t nrows, const uint8_t *chi, const double 
         a.p = b.p = p;
         e64[k] = a;
         e32[k] = b;
-        gidx[p] = k;
         ++k;
     }
 }
@@ -652,7 +618,7 @@ void pd_plan_destroy(pd_plan *p)
 {
     if (!p) return;
     void *ptrs[] = {p->chi, p->chi_om, p->mbits, p->hoff, p->mhat64, p->mhat32, p->ghat64, p->ghat32, p->G64, p->G32,
-                    p->goff, p->gidx, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
+                    p->goff, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
                     p->qt64, p->m3inv64, p->qt32, p->m3inv32, p->tw64, p->tw32, p->spec32, p->spec64,
                     p->work, p->red};
     for (void *q : ptrs)
@@ -1015,10 +981,8 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
         PD_CUDA_TRY(cudaMemcpyAsync(p->goff, cnt.data(), sizeof(int) * (size_t)(nr + 1), cudaMemcpyHostToDevice, st));
         PD_TRY(dalloc(p, &p->gent64, sizeof(GEntry<double>) * (size_t)std::max<int64_t>(acc, 1)));
         PD_TRY(dalloc(p, &p->gent32, sizeof(GEntry<float>) * (size_t)std::max<int64_t>(acc, 1)));
-        PD_TRY(dalloc(p, &p->gidx, sizeof(int) * N));
-        PD_CUDA_TRY(cudaMemsetAsync(p->gidx, 0xff, sizeof(int) * N, st));  // -1
         k_gfill<<<nblk(nr, 128), 128, 0, st>>>(n1, nr, p->chi, p->G64, nc, N, p->goff, (GEntry<double> *)p->gent64,
-                                              (GEntry<float> *)p->gent32, p->gidx);
+                                              (GEntry<float> *)p->gent32);
         PD_LAUNCH_CHECK();
         if (dim == 3 && !pr->fp64 && n1 == n2 && (n1 == 32 || n1 == 64 || n1 == 128)) {
             // FP32 cubes with plane passes: entry -> node, and the per-entry (G p) buffer
@@ -1060,11 +1024,10 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
     }
 
     // twiddles e^{-2 pi i k / L}, L = max(n1, n2, n3), from the eighth-turn symmetric
-    // evaluation of cos/sin in FP64 on the host
+    // evaluation of cos/sin in FP64 on the host, and those of all shorter lengths
     {
         const int L = 1 << p->lgl;
         std::vector<cx<double>> t64(L);
-        std::vector<cx<float>> t32(L);
         for (int k = 0; k < L; ++k) {
             const double a = 2.0 * M_PI * (double)k / (double)L;
             t64[k] = mk(std::cos(a), -std::sin(a));
@@ -1077,11 +1040,21 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
             const double sn[8] = {0, r2, 1, r2, 0, -r2, -1, -r2};
             t64[k] = mk(cs[o], -sn[o]);
         }
-        for (int k = 0; k < L; ++k) t32[k] = mk((float)t64[k].x, (float)t64[k].y);
-        PD_TRY(dalloc(p, &p->tw64, sizeof(cx<double>) * L));
-        PD_TRY(dalloc(p, &p->tw32, sizeof(cx<float>) * L));
-        PD_CUDA_TRY(cudaMemcpyAsync(p->tw64, t64.data(), sizeof(cx<double>) * L, cudaMemcpyHostToDevice, st));
-        PD_CUDA_TRY(cudaMemcpyAsync(p->tw32, t32.data(), sizeof(cx<float>) * L, cudaMemcpyHostToDevice, st));
+        // the tables of every length and stage radix (pd_cols.cuh)
+        const int ne = tw_entries(p->lgl);
+        std::vector<cx<double>> a64(ne, mk(1.0, 0.0));
+        std::vector<cx<float>> a32(ne);
+        for (int k = 0; k <= p->lgl; ++k)
+            for (int r = 0; r < kTwRadices; ++r)
+                for (int i = 0; i < (1 << k) && r <= k; ++i) {
+                    const int e = r ? (i >> r) * (i & ((1 << r) - 1)) : i;  // j q at j 2^r + q
+                    a64[tw_base(k, r) + i] = t64[e << (p->lgl - k)];
+                }
+        for (int i = 0; i < ne; ++i) a32[i] = mk((float)a64[i].x, (float)a64[i].y);
+        PD_TRY(dalloc(p, &p->tw64, sizeof(cx<double>) * ne));
+        PD_TRY(dalloc(p, &p->tw32, sizeof(cx<float>) * ne));
+        PD_CUDA_TRY(cudaMemcpyAsync(p->tw64, a64.data(), sizeof(cx<double>) * ne, cudaMemcpyHostToDevice, st));
+        PD_CUDA_TRY(cudaMemcpyAsync(p->tw32, a32.data(), sizeof(cx<float>) * ne, cudaMemcpyHostToDevice, st));
         PD_CUDA_TRY(cudaStreamSynchronize(st));
     }
 

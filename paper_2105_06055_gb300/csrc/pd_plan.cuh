@@ -7,13 +7,13 @@
 #include <vector>
 
 #include "pd_common.cuh"
+#include "pd_cols.cuh"
 #include "pd_fft.cuh"
+#include "pd_rows.cuh"
 
 namespace pd {
 
-// Packed-spectrum slots per plan. The 3D last-axis pass is out of place: its
-// blocks read the mirror column k2 -> -k2 of another block's tile, so outputs
-// go to slots after the inputs (inputs + outputs <= kMaxSpecFields).
+// Packed-spectrum slots of a plan.
 constexpr int kMaxSpecFields = 20;
 
 // One boundary node of the plan's G field (G != 0 only within delta of the
@@ -58,31 +58,32 @@ struct HorizonDev {
                       // cnt - 1 - c is opposite to bond c)
 };
 
-// Kernel-spectrum lookup from a tile's shared-memory slice (component stride cs)
+// Kernel-spectrum matrix of a mode from its table values (Sym order): the
+// off-diagonal components along folded axes change sign
 template <typename T>
-__device__ __forceinline__ void load_mhat_s(int dim, const T *t, int cs, bool fy, bool fz, T *M /*3x3*/)
+__device__ __forceinline__ void load_mhat_s(int dim, const T *t, bool fy, bool fz, T *M /*3x3*/)
 {
     if (dim == 2) {
-        const T m11 = t[0], m22 = t[cs], m12 = fy ? -t[2 * cs] : t[2 * cs];
+        const T m11 = t[0], m22 = t[1], m12 = fy ? -t[2] : t[2];
         M[0] = m11; M[1] = m12; M[3] = m12; M[4] = m22;
     } else {
-        const T m11 = t[0], m22 = t[cs], m33 = t[2 * cs];
-        const T m12 = fy ? -t[3 * cs] : t[3 * cs];
-        const T m13 = fz ? -t[4 * cs] : t[4 * cs];
-        const T m23 = (fy != fz) ? -t[5 * cs] : t[5 * cs];
+        const T m11 = t[0], m22 = t[1], m33 = t[2];
+        const T m12 = fy ? -t[3] : t[3];
+        const T m13 = fz ? -t[4] : t[4];
+        const T m23 = (fy != fz) ? -t[5] : t[5];
         M[0] = m11; M[1] = m12; M[2] = m13;
         M[3] = m12; M[4] = m22; M[5] = m23;
         M[6] = m13; M[7] = m23; M[8] = m33;
     }
 }
 
-// gamma_i (odd in k_i) from a slice whose components start at t
+// gamma_i (odd in k_i) of a mode from its table values
 template <typename T>
-__device__ __forceinline__ void load_ghat_s(const T *t, int cs, bool fy, bool fz, T *g)
+__device__ __forceinline__ void load_ghat_s(const T *t, bool fy, bool fz, T *g)
 {
     g[0] = t[0];
-    g[1] = fy ? -t[cs] : t[cs];
-    g[2] = fz ? -t[2 * cs] : t[2 * cs];
+    g[1] = fy ? -t[1] : t[1];
+    g[2] = fz ? -t[2] : t[2];
 }
 
 struct LaunchCfg {
@@ -96,7 +97,7 @@ struct pd_plan {
     pd_problem prob;
     int dim, n1, n2, n3, h, ncomp;
     int64_t N, nrows;
-    int lgl;            // log2 twiddle table length
+    int lgl;            // log2 of the longest axis (twiddle tables of all lengths up to it)
     double dV, alpha;   // bond constant (or 30 mu / m0 for the state-based C)
     double ka, m0;      // state-based constants
     double lam_max;     // largest eigenvalue of the periodic symbol
@@ -121,7 +122,6 @@ struct pd_plan {
     double *G64 = nullptr;         // ncomp x N
     float *G32 = nullptr;
     int *goff = nullptr;           // nrows + 1: boundary-node list offsets per row
-    int *gidx = nullptr;           // N: entry of the node in the boundary list, or -1
     int *gnode = nullptr;          // [ngent] node of each boundary entry (plane-pass cubes only)
     void *gpe = nullptr;           // [3][ngent] FP32 (G p) per boundary entry, written by the CG iteration
                                    // while its last-axis pass runs (plane-pass cubes only)
@@ -186,12 +186,12 @@ struct pd_plan {
     int plane_passes = 1;  // FP32 CG on cubes up to 128^3: halves of the iteration whose x1 and x2
                            // transforms run fused in plane passes (bit 0 forward, bit 1 inverse)
     double prof_ms[kKinds] = {};
-    // pass configuration picked by pd_plan_autotune (0: built-in heuristic)
-    int tune_rows = 0;     // rows per row-pass block
-    int tune_w[2] = {0, 0};  // column-tile width of the x2 / last-axis passes
-    int tune_sched = 0;    // FFT stage schedule
-    int tune_stages = 0;   // row-pass pipeline stages (1 or 2; 0: 2)
-    int tune_stages_inv = 0;  // the same for the inverse row passes (0: as tune_stages)
+    // tuning record (pd_plan_tuning; the passes' shapes are constants per length)
+    int tune_rows = 0;
+    int tune_w[2] = {0, 0};
+    int tune_sched = 0;
+    int tune_stages = 0;
+    int tune_stages_inv = 0;
     int energy_direct = 0; // pd_step_verlet: W by a direct horizon sum (pd_plan_set_energy_mode)
     int64_t prof_n[kKinds] = {};
 };
@@ -214,82 +214,6 @@ template <>
 inline const cx<float> *tw_buf<float>(const pd_plan *p) { return p->tw32; }
 template <>
 inline const cx<double> *tw_buf<double>(const pd_plan *p) { return p->tw64; }
-
-// Row-pass configuration: FB packed-row slots, NF node fields of T, NB byte
-// fields; two pipeline stages. c.grid is the tile count; launch_rows caps it
-// at the resident blocks (the kernel is persistent).
-template <typename T>
-inline void row_cfg(const pd_plan *p, int FI, int FB, int NF, int NB, RowGeom &g, LaunchCfg &c)
-{
-    const int H = p->h, nt = H >> kLgV, n1 = 2 * H;
-    const int pad = nt < 16 ? (nt < 2 ? 2 : nt) : 0;  // keeps rows 16-byte aligned, spreads banks
-    const int pitch = H + pad;
-    const int ns_fwd = p->tune_stages == 1 ? 1 : 2;
-    const int ns = (FI > 0 && p->tune_stages_inv > 0) ? p->tune_stages_inv : ns_fwd;
-    auto smem_of = [&](int rows) { return row_smem_bytes<T>(FI, FB, NF, NB, rows, pitch, n1, ns); };
-    int rows = p->tune_rows > 0 ? p->tune_rows : 128 / nt;
-    if (rows < 1) rows = 1;
-    // whole warps: the epilogues' block reductions shuffle over full warps
-    // (the heuristic and the autotuner never go below; a pinned value could)
-    if (rows * nt < 32) rows = 32 / nt;
-    while (rows > 1 && rows * nt > 256) rows >>= 1;  // k_rows launch bound
-    while (rows > 1 && smem_of(rows) > 100 * 1024) rows >>= 1;
-    while (p->nrows % rows) rows >>= 1;
-    g.lgh = ilog2(H);
-    g.rows = rows;
-    g.pitch = pitch;
-    g.nrows = p->nrows;
-    g.lgl = p->lgl;
-    g.sched = p->tune_sched;
-    g.nstage = ns;
-    g.err = p->dev_status;
-    g.inject = p->inject;
-    c.grid = dim3((unsigned)(p->nrows / rows));
-    c.block = dim3(rows * nt);
-    c.smem = smem_of(rows);
-}
-
-// Column-pass configuration: axis 1 = x2, axis 2 = x3 (3D); FB fields in the
-// tile, FI of them with a mirror column. The 3D last-axis pass runs as two
-// launches with one tile width: tmode 1 (tiles without kx = 0: no mirror
-// column, no kx = n1/2 table column) and tmode 2 (the kx = 0 tile of each k2
-// row, with the mirror column of -k2).
-template <typename T>
-inline void col_cfg(const pd_plan *p, int axis, bool last, int FB, int FI, int NTAB, int tmode, ColGeom &g,
-                    LaunchCfg &c, int64_t &inner)
-{
-    const int H = p->h;
-    const int L = axis == 1 ? p->n2 : p->n3;
-    const int nt = L >> kLgV;
-    const bool split = p->dim == 3 && last;
-    const int wmirror = split ? 1 : 0;  // the width must also fit the kx = 0 tiles
-    const int mirror = (tmode == 2 || (split && tmode == 0)) ? 1 : 0;  // tmode 0 + split: one launch, all tiles
-    inner = axis == 1 ? (int64_t)H : (int64_t)p->n2 * H;
-    auto smem_of = [&](int w, int mir, int tc) {
-        const size_t tab = (((size_t)NTAB * (L / 2 + 1) * tc + 1) & ~(size_t)1) * sizeof(T);
-        return (size_t)L * sizeof(cx<T>) + (size_t)FB * L * w * sizeof(cx<T>) +
-               (mir ? (size_t)FB * L * 2 * sizeof(cx<T>) : 0) + tab + 8 * ((size_t)FB + 1);
-    };
-    int w = p->tune_w[last ? 1 : 0] > 0 ? p->tune_w[last ? 1 : 0] : 32;
-    while (w > 2 && ((w + wmirror) * nt > 512 || smem_of(w, wmirror, w + 1) > 100 * 1024 || (H % w))) w >>= 1;
-    g.lgl = ilog2(L);
-    g.w = w;
-    g.lgw = ilog2(w);
-    g.mirror = mirror;
-    g.lgh = ilog2(H);
-    g.n2 = p->n2;
-    g.lgtw = p->lgl;
-    g.lb = L < 256 ? L : 256;
-    g.outer = axis == 1 ? p->n3 : 1;
-    g.sched = p->tune_sched;
-    g.tmode = split ? tmode : 0;
-    g.err = p->dev_status;
-    unsigned gx = (unsigned)(inner / w);
-    if (split && tmode != 0) gx = tmode == 2 ? (unsigned)p->n2 : (unsigned)(p->n2 * (H / w - 1));
-    c.grid = dim3(gx, (unsigned)g.outer);
-    c.block = dim3((w + mirror) * nt);
-    c.smem = smem_of(w, mirror, w + (split && tmode == 1 ? 0 : 1));
-}
 
 pd_status set_smem_attr(const void *func, size_t smem);
 
@@ -362,52 +286,62 @@ inline pd_status launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 bloc
     return PD_OK;
 }
 
-// Row ops that declare kFixedLength = true also get row kernels compiled for
-// the packed row lengths of the 128^3 to 512^3 boxes (64 to 256 values), one
-// per stage schedule where the schedule matters; other lengths use the kernel
-// that reads the length at run time.
-template <class Op, class = void>
-struct op_fixed_len : std::false_type {
-};
-template <class Op>
-struct op_fixed_len<Op, std::void_t<decltype(Op::kFixedLength)>> : std::bool_constant<Op::kFixedLength> {
-};
-
+// Row kernels are compiled per row length, with the index arithmetic as
+// constants (at 128^3 the forward pass: 28 us with the length read at run time, 16
+// us so), for boxes of 64 to 2048 nodes along x1 in 2D and 32 to 512 in 3D; the
+// remaining lengths share one kernel that reads it.
 template <typename T, class Op>
-auto rows_kernel(int lgh, int sched)
+auto rows_kernel(int lgh)
 {
     using K = decltype(&k_rows<T, Op>);
-    if constexpr (op_fixed_len<Op>::value) {
+    if constexpr (Op::kDim == 2) {
         switch (lgh) {
-            case 6: return (K)&k_rows<T, Op, 6, 0>;
-            case 7: return sched ? (K)&k_rows<T, Op, 7, 1> : (K)&k_rows<T, Op, 7, 0>;
-            case 8: return sched ? (K)&k_rows<T, Op, 8, 1> : (K)&k_rows<T, Op, 8, 0>;
+            case 9: return (K)&k_rows<T, Op, 9>;
+            case 10: return (K)&k_rows<T, Op, 10>;
             default: break;
         }
+    } else if (lgh == 4) {
+        return (K)&k_rows<T, Op, 4>;
+    }
+    switch (lgh) {
+        case 5: return (K)&k_rows<T, Op, 5>;
+        case 6: return (K)&k_rows<T, Op, 6>;
+        case 7: return (K)&k_rows<T, Op, 7>;
+        case 8: return (K)&k_rows<T, Op, 8>;
+        default: break;
     }
     return (K)&k_rows<T, Op>;
 }
 
-// Persistent row pass: as many blocks as fit on the GPU at once (at most one
-// per tile). *grid_out receives the block count (the number of block partial
-// sums an op with a block accumulator writes).
+// Row pass: tile and warps by row_tile_rows and row_warps (fewer rows when the
+// grid has fewer). Passes with block reductions run on at most 8 blocks per SM
+// (each block writes partial sums), the others on a block per tile. *grid_out
+// receives the block count.
 template <typename T, class Op>
 pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_out = nullptr)
 {
+    constexpr int FB = Op::kFin > Op::kFout ? Op::kFin : Op::kFout;
     RowGeom g;
-    LaunchCfg c;
-    constexpr int KO = Op::kFout > Op::kStage ? Op::kFout : Op::kStage;
-    constexpr int FB = Op::kFin > KO ? Op::kFin : KO;
-    row_cfg<T>(p, Op::kFin, FB, Op::kNF, Op::kNB, g, c);
-    const auto kern = rows_kernel<T, Op>(g.lgh, g.sched);
-    PD_TRY(set_smem_attr((const void *)kern, c.smem));
-    int per_sm = 0;
-    PD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)c.block.x, c.smem));
-    const int64_t cap = (int64_t)std::max(per_sm, 1) * p->nsm;
-    if ((int64_t)c.grid.x > cap) c.grid.x = (unsigned)cap;
-    if (grid_out) *grid_out = c.grid.x;
+    g.lgh = ilog2(p->h);
+    g.rows = row_tile_rows(p->h, FB);
+    bool whole = true;  // the tile size the fixed-length kernels are compiled for
+    while (p->nrows % g.rows) {
+        g.rows >>= 1;
+        whole = false;
+    }
+    g.nrows = p->nrows;
+    g.err = p->dev_status;
+    g.inject = p->inject;
+    const size_t smem =
+        16 + (size_t)Op::kNB * g.rows * p->n1 + (size_t)FB * g.rows * row_pitch(p->h) * sizeof(cx<T>);
+    int64_t grid = p->nrows / g.rows;
+    if (op_reduce<Op>::value) grid = std::min<int64_t>(grid, 8 * (int64_t)p->nsm);
+    if (grid_out) *grid_out = (unsigned)grid;
+    const auto kern = whole ? rows_kernel<T, Op>(g.lgh) : &k_rows<T, Op>;
+    PD_TRY(set_smem_attr((const void *)kern, smem));
     PD_TRY(prof_begin(p, Op::kFin > 0 ? PASS_ROWS_INV : PASS_ROWS_FWD, st));
-    PD_TRY(launch_k(p->pdl != 0, kern, c.grid, c.block, c.smem, st, g, op, tw_buf<T>(p)));
+    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(FB)), smem, st, g, op,
+                    tw_buf<T>(p)));
     PD_TRY(prof_end(p, st));
     p->launches++;
     return PD_OK;
@@ -416,83 +350,72 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
 template <typename T>
 inline int spec_slots(const pd_plan *p) { return sizeof(T) == 8 ? p->spec64_slots : p->spec32_slots; }
 
-template <class Op>
-constexpr int op_tab()
+// Geometry of a column pass along x2 (zaxis 0) or x3 (zaxis 1).
+template <typename T>
+inline ColArgs<T> col_args(const pd_plan *p, int zaxis)
 {
-    if constexpr (Op::kMode == 2)
-        return Op::kTab;
-    else
-        return 0;
+    ColArgs<T> g;
+    g.spec = reinterpret_cast<cx<T> *>(const_cast<T *>(spec_buf<T>(p)));
+    g.fs = p->N / 2;
+    g.ls = zaxis ? (int64_t)p->n2 * p->h : (int64_t)p->h;
+    g.os = (int64_t)p->n2 * p->h;
+    g.lgh = ilog2(p->h);
+    g.n2 = zaxis ? p->n2 : 1;
+    g.nspec = 0;
+    g.zaxis = zaxis;
+    return g;
 }
 
+template <typename T, int LG, bool INV>
+pd_status launch_plain(pd_plan *p, int slot0, int fields, cudaStream_t st)
+{
+    using S = PlainShape<T, LG, INV>;
+    const auto kern = k_col_plain<T, LG, INV>;
+    PD_TRY(set_smem_attr((const void *)kern, S::smem));
+    return launch_k(p->pdl != 0, kern, dim3((unsigned)(p->h / S::W), (unsigned)p->n3, (unsigned)fields),
+                    dim3(S::THREADS), S::smem, st, col_args<T>(p, 0), slot0, tw_buf<T>(p));
+}
+
+// Plain transforms along x2 of the spectra in slots slot0 ... slot0 + fields - 1, in place.
+template <typename T>
+pd_status col_pass(pd_plan *p, int slot0, int fields, bool inverse, cudaStream_t st);
+
+template <typename T, class Op, int LG>
+pd_status launch_comb_lg(pd_plan *p, const Op &op, cudaStream_t st)
+{
+    using S = CombShape<T, Op, LG>;
+    const auto kern = k_col_comb<T, Op, LG>;
+    PD_TRY(set_smem_attr((const void *)kern, S::smem));
+    const int z = p->dim == 3 ? 1 : 0;
+    ColArgs<T> g = col_args<T>(p, z);
+    // pairs of kx = 0 columns: k2 = 0 ... n2/2 in 3D, one column in 2D
+    constexpr int sw = S::W < kSpecCols ? S::W : kSpecCols;
+    g.nspec = ((z ? p->n2 + 2 : 2) + sw - 1) / sw;
+    const unsigned tiles = (unsigned)((int64_t)(z ? p->n2 : 1) * p->h / S::W);
+    return launch_k(p->pdl != 0, kern, dim3(tiles + (unsigned)g.nspec), dim3(S::THREADS), S::smem, st, g, op,
+                    tw_buf<T>(p));
+}
+
+// The last-axis pass: forward transform, spectral combine, inverse transform.
 template <typename T, class Op>
-pd_status launch_cols(pd_plan *p, const Op &op, int axis, bool last, int F, cudaStream_t st)
+pd_status launch_comb(pd_plan *p, const Op &op, cudaStream_t st)
 {
-    // The 3D last-axis pass runs as two launches: the kx = 0 tiles (one per k2
-    // row, with the mirror column) on the plan's second stream beside the
-    // other tiles on `st` (fork and join by events; inside a stream capture
-    // they become parallel graph branches). Bodies of conditional graph nodes
-    // are captured from one stream only (no_fork): there the two launches
-    // follow each other.
-    const bool split = p->dim == 3 && last;
-    const bool fork = split && p->aux_stream && !p->no_fork;
-    PD_TRY(prof_begin(p, last ? PASS_LAST : PASS_COLS, st));
-    if (fork) {
-        PD_CUDA_TRY(cudaEventRecord(p->ev_fork[0], st));
-        PD_CUDA_TRY(cudaStreamWaitEvent(p->aux_stream, p->ev_fork[0], 0));
+    PD_TRY(prof_begin(p, PASS_LAST, st));
+    pd_status s = PD_ERR_SIZE;
+    switch (ilog2(p->dim == 3 ? p->n3 : p->n2)) {
+        case 4: s = launch_comb_lg<T, Op, 4>(p, op, st); break;
+        case 5: s = launch_comb_lg<T, Op, 5>(p, op, st); break;
+        case 6: s = launch_comb_lg<T, Op, 6>(p, op, st); break;
+        case 7: s = launch_comb_lg<T, Op, 7>(p, op, st); break;
+        case 8: s = launch_comb_lg<T, Op, 8>(p, op, st); break;
+        case 9: s = launch_comb_lg<T, Op, 9>(p, op, st); break;
+        case 10: s = launch_comb_lg<T, Op, 10>(p, op, st); break;
+        default: set_error("axis length outside 16..1024"); break;
     }
-    for (int tmode = split ? 2 : 0; tmode >= (split ? 1 : 0); --tmode) {
-        cudaStream_t ls = (fork && tmode == 2) ? p->aux_stream : st;
-        ColGeom g;
-        LaunchCfg c;
-        int64_t inner = 0;
-        col_cfg<T>(p, axis, last, F, Op::kFin, Op::kMode == 2 ? op_tab<Op>() : 0, tmode, g, c, inner);
-        if (c.grid.x == 0) continue;  // one tile per k2 row: no tmode-1 tiles
-        const int L = 1 << g.lgl;
-        const unsigned long long dims[3] = {(unsigned long long)(2 * inner), (unsigned long long)L,
-                                            (unsigned long long)g.outer * spec_slots<T>(p)};
-        const unsigned long long strides[2] = {(unsigned long long)(2 * inner * sizeof(T)),
-                                               (unsigned long long)(2 * inner * L * sizeof(T))};
-        const unsigned box_t[3] = {(unsigned)(2 * g.w), (unsigned)g.lb, 1u};
-        const unsigned box_m[3] = {4u, (unsigned)g.lb, 1u};
-        CUtensorMap tmt, tmm;
-        PD_TRY(encode_tmap_3d(&tmt, spec_buf<T>(p), sizeof(T) == 8, dims, strides, box_t));
-        PD_TRY(encode_tmap_3d(&tmm, spec_buf<T>(p), sizeof(T) == 8, dims, strides, box_m));
-        PD_TRY(set_smem_attr((const void *)k_cols<T, Op>, c.smem));
-        PD_TRY(launch_k(p->pdl != 0, k_cols<T, Op>, c.grid, c.block, c.smem, ls, g, op, tw_buf<T>(p),
-                        axis == 2 ? 1 : 0, tmt, tmm));
-        p->launches++;
-    }
-    if (fork) {
-        PD_CUDA_TRY(cudaEventRecord(p->ev_fork[1], p->aux_stream));
-        PD_CUDA_TRY(cudaStreamWaitEvent(st, p->ev_fork[1], 0));
-    }
+    PD_TRY(s);
     PD_TRY(prof_end(p, st));
+    p->launches++;
     return PD_OK;
-}
-
-// Plain column FFT of F packed spectra (slots slot0 ... slot0+F-1) along x2, in place.
-template <typename T, int F, int MODE>
-struct ColPass {
-    static constexpr int kFin = F, kFout = F, kMode = MODE, kPre = 0, kTab = 0;
-    static constexpr bool kStoreIn = false;
-    int slot0;
-    __device__ int slot_in(int f) const { return slot0 + f; }
-    __device__ int slot_out(int f) const { return slot0 + f; }
-    __device__ int slot_aux(int) const { return 0; }
-    __device__ const T *table(int) const { return nullptr; }
-    __device__ void combine(const T *, int, bool, bool, const cx<T> *, cx<T> *) const {}
-};
-
-template <typename T, int F>
-pd_status col_pass(pd_plan *p, int slot0, bool inverse, cudaStream_t st)
-{
-    if (inverse) {
-        ColPass<T, F, 1> op{slot0};
-        return launch_cols<T>(p, op, 1, false, F, st);
-    }
-    ColPass<T, F, 0> op{slot0};
-    return launch_cols<T>(p, op, 1, false, F, st);
 }
 
 }  // namespace pd

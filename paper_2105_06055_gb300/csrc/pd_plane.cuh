@@ -7,7 +7,7 @@
 // owns one field of one x3-plane and runs both transforms on the plane in
 // shared memory, so each CG iteration is
 //   plane forward  : CG vector update, chi p, x1 R2C, x2 FFT      (one kernel)
-//   last axis      : x3 FFT, spectral multiply, inverse x3 FFT   (k_cols)
+//   last axis      : x3 FFT, spectral multiply, inverse x3 FFT   (k_col_comb)
 //   G p            : (G p) per boundary-list entry   (k_gp_entries, beside the last axis)
 //   plane inverse  : x2 inverse FFT, x1 C2R, L = chi y - G p, q, inner products
 //   finish         : alpha, beta
@@ -39,15 +39,13 @@ template <typename T>
 struct PlaneArgs {
     T *e, *r, *pv, *q;      // CG vectors: D components of N nodes each
     const uint8_t *bits;    // per node: bit 0 chi, bit 1 + i chi_Omega of component i
-    cx<T> *spec;            // spectrum slots (fs complex each): the forward pass writes slots
-                            // 0..D-1, the inverse pass reads slots D..2D-1
+    cx<T> *spec;            // spectrum slots (fs complex each): slots 0..D-1
     int64_t fs, N;
     double *red;            // reduction buffer: partials and scalars
     const T *gpe;           // [D][nent] (G p) per boundary-list entry (k_gp_entries)
     const int *gnode;       // [nent] node of each entry
     const int *goff;        // per row: first entry of the row (nrows + 1 offsets; the list is ordered by node)
     int64_t nent;
-    int lgl;                // log2 of the plan's twiddle table length
     int *err;               // device status word
     int *inject;            // failure-handling test hook (see k_rows): kind 5 stalls the inverse plane pass
 };
@@ -135,7 +133,7 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
     cx<T> *pl = reinterpret_cast<cx<T> *>(smem_raw + S::kTw);
     const int tid = threadIdx.x;
     const int j = blockIdx.x % D, z = blockIdx.x / D;
-    for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[i << (a.lgl - S::LGT)];
+    for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[tw_base(S::LGT, 0) + i];
     pdl_wait();
     pdl_trigger();
 
@@ -220,7 +218,7 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
     const int j = blockIdx.x % D, z = blockIdx.x / D;
     const int64_t pbase = (int64_t)z * S::n2 * S::n1;  // first node of the plane
     if (tid == 0) mbar_init(mbar, 1);
-    for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[i << (a.lgl - S::LGT)];
+    for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[tw_base(S::LGT, 0) + i];
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -228,7 +226,7 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
         // test hook: one-shot, so a pass captured in a graph stalls on one replay only
         const bool stall = a.inject && blockIdx.x == 0 && atomicCAS(a.inject, 6, 0) == 6;
         if (!stall) {
-            const cx<T> *src = a.spec + (int64_t)(D + j) * a.fs + (int64_t)z * S::n2 * S::H;
+            const cx<T> *src = a.spec + (int64_t)j * a.fs + (int64_t)z * S::n2 * S::H;
             mbar_expect_tx(mbar, (unsigned)(S::n2 * S::H * sizeof(cx<T>)));
             for (int y = 0; y < S::n2; ++y)
                 bulk_load(pl + y * S::PITCH, src + (int64_t)y * S::H, S::H * sizeof(cx<T>), mbar);

@@ -143,13 +143,11 @@ __global__ void k_cg_q(T *q, const T *pp, const uint8_t *co, int64_t n, double *
 }
 
 // rows, forward: pending update e += alpha p, r -= alpha q, then
-// p = r + beta p (stored), partials of r.r, transform chi p. Node fields come
-// straight from global memory (coalesced pairs); only the mask bits are staged.
+// p = r + beta p (stored), partials of r.r, transform chi p
 template <typename T, int D>
 struct ProCG {
-    static constexpr int kFin = 0, kFout = D, kNF = 0, kNB = 1, kStage = 0;
-    static constexpr bool kSparse = false, kNodeAcc = true;
-    static constexpr bool kFixedLength = std::is_same_v<T, float>;
+    static constexpr int kFin = 0, kFout = D, kNB = 1, kDim = D;
+    static constexpr bool kReduce = true;
     T *e, *r, *pv;
     const T *q;
     const uint8_t *bits;
@@ -160,80 +158,59 @@ struct ProCG {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int) const { return nullptr; }
     __device__ cx<T> *spec_out(int f) const { return spec + f * fstride; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return bits; }
-    // e, r, p and q of the tile's rows start towards L2 while its mask bytes arrive
-    __device__ __forceinline__ void l2_prefetch(int64_t row0, int rows) const
+    struct Nd {
+        typename vec2<T>::type ee[D], rr[D], pp[D], qq[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        const int64_t base = row0 * n1;
-        const unsigned bytes = (unsigned)(rows * n1 * sizeof(T));
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            bulk_prefetch_l2(e + j * N + base, bytes);
-            bulk_prefetch_l2(r + j * N + base, bytes);
-            bulk_prefetch_l2(pv + j * N + base, bytes);
-            bulk_prefetch_l2(q + j * N + base, bytes);
+            nd.ee[j] = load2(e + (j * N + p0) + o);
+            nd.rr[j] = load2(r + (j * N + p0) + o);
+            nd.pp[j] = load2(pv + (j * N + p0) + o);
+            nd.qq[j] = load2(q + (j * N + p0) + o);
         }
     }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *, const T *, T *o0,
-                                          T *o1, DSum &acc) const
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *, const T *, T *o0, T *o1,
+                                          DSum &acc) const
     {
         const double *s = red + kRedScal;
         const T alpha = (T)s[S_ALPHA], beta = (T)s[S_BETA];
-        const T v0 = (c.b(0, rl, i1) & 1) ? T(1) : T(0), v1 = (c.b(0, rl, i1 + 1) & 1) ? T(1) : T(0);
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        typename vec2<T>::type ee[D], rr[D], pp[D], qq[D];
+        T v0, v1;
+        chi_pair(c, o, v0, v1);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            ee[j] = load2(e + j * N + p);
-            rr[j] = load2(r + j * N + p);
-            pp[j] = load2(pv + j * N + p);
-            qq[j] = load2(q + j * N + p);
-        }
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            store2(e + j * N + p, ee[j].x + alpha * pp[j].x, ee[j].y + alpha * pp[j].y);
-            const T ra = rr[j].x - alpha * qq[j].x, rb = rr[j].y - alpha * qq[j].y;
-            store2(r + j * N + p, ra, rb);
+            store2(e + (j * N + c.p0) + o, nd.ee[j].x + alpha * nd.pp[j].x, nd.ee[j].y + alpha * nd.pp[j].y);
+            const T ra = nd.rr[j].x - alpha * nd.qq[j].x, rb = nd.rr[j].y - alpha * nd.qq[j].y;
+            store2(r + (j * N + c.p0) + o, ra, rb);
             acc.add_prod(ra, ra);
             acc.add_prod(rb, rb);
-            const T a = ra + beta * pp[j].x;
-            const T b = rb + beta * pp[j].y;
-            store2(pv + j * N + p, a, b);
+            const T a = ra + beta * nd.pp[j].x;
+            const T b = rb + beta * nd.pp[j].y;
+            store2(pv + (j * N + c.p0) + o, a, b);
             o0[j] = v0 * a;
             o1[j] = v1 * b;
         }
     }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ void emit(const RowCtx<T> &, int, int, const T *, const T *, DSum &) const {}
     __device__ void block_done(DSum &acc) const { write_partial(red, acc); }
 };
-
-static_assert(op_min_blocks<ProCG<float, 3>>::value == 1, "ProCG declares no register cap");
 
 struct CgAcc {
     DSum pq, rq, qq;
 };
 
-// rows, inverse: L = chi y - G p (G from the boundary list, looked up per node
-// with the p already in registers), q = -chi_O L, block partials of p.q,
-// r.q, q.q
+// rows, inverse: L = chi (y - G p) (G from the boundary list), q = -chi_O L, block
+// partials of p.q, r.q, q.q
 template <typename T, int D>
 struct EpiCG {
-    static constexpr int kFin = D, kFout = 0, kStage = D, kNF = 0, kNB = 1;
-    static constexpr bool kSparse = false;
-    static constexpr bool kFixedLength = std::is_same_v<T, float>;
-    static constexpr int kMinBlocks = 4;  // <= 64 registers: more resident warps
+    static constexpr int kFin = D, kFout = 0, kNB = 1, kDim = D;
+    static constexpr bool kReduce = true, kEntries = true;
     using Acc = CgAcc;
-    // loads of one node pair: p, r and its boundary-list indices (read-only in this pass)
-    struct EmitIn {
-        typename vec2<T>::type pp[D], rr[D];
-        int2 gi;
-    };
     const T *pv, *r;
     const uint8_t *bits;
     const GEntry<T> *gent;
-    const int *gidx;
+    const int *goff;
     T *q;
     double *red;
     int64_t N;
@@ -242,98 +219,49 @@ struct EpiCG {
     int64_t fstride;
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
-    __device__ const T *nf_src(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return bits; }
-    // p, r and the boundary index of the tile's rows start towards L2 while
-    // the tile's spectra arrive and are transformed (one bulk prefetch each)
-    __device__ __forceinline__ void l2_prefetch(int64_t row0, int rows) const
+    __device__ __forceinline__ const int *rows_off() const { return goff; }
+    __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {
-        const int64_t base = row0 * n1;
-        const unsigned bytes = (unsigned)(rows * n1 * sizeof(T));
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            bulk_prefetch_l2(pv + j * N + base, bytes);
-            bulk_prefetch_l2(r + j * N + base, bytes);
-        }
-        bulk_prefetch_l2(gidx + base, (unsigned)(rows * n1 * sizeof(int)));
-    }
-    __device__ __forceinline__ void node2(const RowCtx<T> &c, int rl, int i1, const T *in0, const T *in1, T *o0,
-                                          T *o1) const
-    {
-        const T v0 = (c.b(0, rl, i1) & 1) ? T(1) : T(0), v1 = (c.b(0, rl, i1 + 1) & 1) ? T(1) : T(0);
+        const GEntry<T> e = gent[k];
+        p = e.p;
+        T x[D], y[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            o0[i] = v0 * in0[i];
-            o1[i] = v1 * in1[i];
+            x[i] = pv[i * N + p];
+            y[i] = T(0);
         }
+        sym_apply<T, D>(e.g, x, y);
+#pragma unroll
+        for (int i = 0; i < D; ++i) s[i] = -y[i];
     }
-    __device__ void sparse(const RowCtx<T> &, int, int) const {}
-    __device__ __forceinline__ void load_emit(const RowCtx<T> &c, int rl, int i1, EmitIn &in) const
+    struct Nd {
+        T pa[D], pb[D], ra[D], rb[D];
+    };
+    __device__ __forceinline__ void load(Nd &nd, int64_t p0, int o) const
     {
-        using V = typename vec2<T>::type;
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        in.gi = __ldg(reinterpret_cast<const int2 *>(gidx + p));
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            in.pp[i] = __ldg(reinterpret_cast<const V *>(pv + i * N + p));
-            in.rr[i] = __ldg(reinterpret_cast<const V *>(r + i * N + p));
+            load_pair(pv + (i * N + p0) + o, nd.pa[i], nd.pb[i]);
+            load_pair(r + (i * N + p0) + o, nd.ra[i], nd.rb[i]);
         }
     }
-    __device__ __forceinline__ void emit(const RowCtx<T> &c, int rl, int i1, const T *s0, const T *s1,
-                                         CgAcc &acc) const
+    __device__ __forceinline__ void node2(const RowCtx &c, int o, Nd &nd, const T *in0, const T *in1, T *, T *,
+                                          CgAcc &acc) const
     {
-        EmitIn in;
-        load_emit(c, rl, i1, in);
-        emit_loaded(c, rl, i1, s0, s1, acc, in);
-    }
-    __device__ __forceinline__ void emit_loaded(const RowCtx<T> &c, int rl, int i1, const T *s0, const T *s1,
-                                                CgAcc &acc, const EmitIn &in) const
-    {
-        const int64_t p = (c.row0 + rl) * n1 + i1;
-        const unsigned b0 = c.b(0, rl, i1), b1 = c.b(0, rl, i1 + 1);
-        const int2 gi = in.gi;
-        const typename vec2<T>::type *pp = in.pp, *rr = in.rr;
-        T L0[D], L1[D];
+        const uchar2 b = c.b2(0, o);
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            L0[i] = s0[i];
-            L1[i] = s1[i];
-        }
-        if (gi.x >= 0) {
-            const GEntry<T> e = gent[gi.x];
-            T x[D], y[D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
-                x[i] = pp[i].x;
-                y[i] = T(0);
-            }
-            sym_apply<T, D>(e.g, x, y);
-#pragma unroll
-            for (int i = 0; i < D; ++i) L0[i] -= y[i];
-        }
-        if (gi.y >= 0) {
-            const GEntry<T> e = gent[gi.y];
-            T x[D], y[D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
-                x[i] = pp[i].y;
-                y[i] = T(0);
-            }
-            sym_apply<T, D>(e.g, x, y);
-#pragma unroll
-            for (int i = 0; i < D; ++i) L1[i] -= y[i];
-        }
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const T a = ((b0 >> (1 + i)) & 1) ? -L0[i] : T(0);
-            const T b = ((b1 >> (1 + i)) & 1) ? -L1[i] : T(0);
-            store2(q + i * N + p, a, b);
-            acc.pq.add_prod(pp[i].x, a);
-            acc.pq.add_prod(pp[i].y, b);
-            acc.rq.add_prod(rr[i].x, a);
-            acc.rq.add_prod(rr[i].y, b);
-            acc.qq.add_prod(a, a);
-            acc.qq.add_prod(b, b);
+            const T L0 = (b.x & 1) ? in0[i] : T(0), L1 = (b.y & 1) ? in1[i] : T(0);
+            const T x = ((b.x >> (1 + i)) & 1) ? -L0 : T(0);
+            const T y = ((b.y >> (1 + i)) & 1) ? -L1 : T(0);
+            store2(q + (i * N + c.p0) + o, x, y);
+            acc.pq.add_prod(nd.pa[i], x);
+            acc.pq.add_prod(nd.pb[i], y);
+            acc.rq.add_prod(nd.ra[i], x);
+            acc.rq.add_prod(nd.rb[i], y);
+            acc.qq.add_prod(x, x);
+            acc.qq.add_prod(y, y);
         }
     }
     __device__ void block_done(CgAcc &acc) const
@@ -349,9 +277,6 @@ struct EpiCG {
         }
     }
 };
-
-static_assert(op_min_blocks<EpiCG<float, 3>>::value == EpiCG<float, 3>::kMinBlocks,
-              "the row kernel must apply the epilogue's register cap");
 
 // log2(n1 / 2) when the plane passes apply (FP32 cubes of 32^3, 64^3 or 128^3:
 // one field of an x1-x2 plane fits in shared memory), else 0
@@ -467,25 +392,24 @@ struct Solver {
         const int64_t fs = p->N / 2;
         const Model<T> m = model_view<T>(p);
         unsigned gpro = 0, gepi = 0;
-        const int ob = D == 3 ? D : 0;
-        const int lgh = plane_lgh<T, D>(p);
+            const int lgh = plane_lgh<T, D>(p);
         const bool plane_fwd = lgh && (p->plane_passes & 1), plane_inv = lgh && (p->plane_passes & 2);
         const PlaneArgs<T> pa{e, r, pv, q, p->mbits, spec, fs, p->N, p->red, (const T *)p->gpe, p->gnode, p->goff,
-                              p->ngent, p->lgl, p->dev_status, p->inject};
+                              p->ngent, p->dev_status, p->inject};
         if (plane_fwd) {
             PD_TRY((plane_pass<T, D>(lgh, true, pa)));
             gpro = (unsigned)(D * p->n3);
         } else {
             ProCG<T, D> pro{e, r, pv, q, p->mbits, p->red, p->N, p->n1, spec, fs};
             PD_TRY(launch_rows<T>(p, pro, st, &gpro));
-            if (D == 3) PD_TRY((col_pass<T, D>(p, 0, false, st)));
+            if (D == 3) PD_TRY(col_pass<T>(p, 0, D, false, st));
         }
+        const bool gp_fork = plane_inv && p->ngent > 0 && p->aux_stream && !p->no_fork;
         if (plane_inv && p->ngent > 0) {
             // (G p) per boundary entry for the inverse plane pass, on the second
-            // stream beside the last-axis pass (joined by that pass's join)
-            const bool fork = p->aux_stream && !p->no_fork;
-            cudaStream_t gs = fork ? p->aux_stream : st;
-            if (fork) {
+            // stream beside the last-axis pass
+            cudaStream_t gs = gp_fork ? p->aux_stream : st;
+            if (gp_fork) {
                 PD_CUDA_TRY(cudaEventRecord(p->ev_fork[0], st));
                 PD_CUDA_TRY(cudaStreamWaitEvent(gs, p->ev_fork[0], 0));
             }
@@ -493,15 +417,17 @@ struct Solver {
             k_gp_entries<T, D><<<gb, 256, 0, gs>>>(m.gent, p->ngent, (const T *)pv, p->N, (T *)p->gpe);
             PD_LAUNCH_CHECK();
             p->launches++;
+            if (gp_fork) PD_CUDA_TRY(cudaEventRecord(p->ev_fork[1], gs));
         }
-        CombForce<T, D, false> cmb{m, ob};
-        PD_TRY(launch_cols<T>(p, cmb, D == 3 ? 2 : 1, true, D, st));
+        CombForce<T, D, false> cmb{m};
+        PD_TRY(launch_comb<T>(p, cmb, st));
+        if (gp_fork) PD_CUDA_TRY(cudaStreamWaitEvent(st, p->ev_fork[1], 0));
         if (plane_inv) {
             PD_TRY((plane_pass<T, D>(lgh, false, pa)));
             gepi = (unsigned)(D * p->n3);
         } else {
-            if (D == 3) PD_TRY((col_pass<T, D>(p, ob, true, st)));
-            EpiCG<T, D> epi{pv, r, p->mbits, m.gent, p->gidx, q, p->red, p->N, p->n1, spec + ob * fs, fs};
+            if (D == 3) PD_TRY(col_pass<T>(p, 0, D, true, st));
+            EpiCG<T, D> epi{pv, r, p->mbits, m.gent, p->goff, q, p->red, p->N, p->n1, spec, fs};
             PD_TRY(launch_rows<T>(p, epi, st, &gepi));
         }
         if (gpro > (unsigned)kPartB || gepi > (unsigned)kPartB) {

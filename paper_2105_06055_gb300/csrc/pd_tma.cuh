@@ -1,13 +1,10 @@
-// Tensor Memory Accelerator (TMA) and mbarrier helpers for sm_103a (private).
+// Bulk asynchronous copies and mbarrier helpers for sm_103a (private).
 //
-// Tiles move between global and shared memory with cp.async.bulk.tensor
-// (loads complete on an mbarrier, stores drain through a bulk group), issued by
-// one thread per block; the rest of the block only waits. Every wait on an
-// mbarrier is bounded by the global timer: on time-out the block sets a bit in
-// the plan's device status word and leaves without touching the tile.
+// Rows move between global and shared memory with cp.async.bulk (loads complete
+// on an mbarrier, stores drain through a bulk group). Every wait on an mbarrier
+// is bounded by the global timer: on time-out the block sets a bit in the plan's
+// device status word and leaves without touching the tile.
 #pragma once
-
-#include <cuda.h>
 
 #include "pd_common.cuh"
 
@@ -68,22 +65,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, unsigned pha
     return true;
 }
 
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *m, int x, int y, int z,
-                                            unsigned long long *mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_u32(dst)), "l"(m), "r"(x), "r"(y), "r"(z), "r"(smem_u32(mbar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, int x, int y, int z, const void *src)
-{
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(m),
-                 "r"(x), "r"(y), "r"(z), "r"(smem_u32(src))
-                 : "memory");
-}
-
 // 1D bulk copy global -> shared (16-byte aligned addresses, size multiple of 16)
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *mbar)
 {
@@ -119,10 +100,5 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // make this thread's generic-proxy shared-memory writes visible to the async proxy
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Host: encode a 3D tiled tensor map (dims/box in elements, dim 0 innermost;
-// strides in bytes for dims 1 and 2).
-pd_status encode_tmap_3d(CUtensorMap *m, void *base, bool fp64, const unsigned long long dims[3],
-                         const unsigned long long strides[2], const unsigned box[3]);
 
 }  // namespace pd

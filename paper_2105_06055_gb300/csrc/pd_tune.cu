@@ -1,25 +1,17 @@
-// Autotuner for the FFT passes: picks, per plan, the rows per block of the
-// row passes and their pipeline depth (one or two shared-memory stages), the
-// tile width of the column passes (x2 and last axis) and the FFT stage
-// schedule (radix-4/2 remainder stage first or last) by timing the plan's own
-// force evaluation (pd_plan_autotune) or a chunk of its static solver's CG
-// iterations (pd_plan_autotune_solve) on its workspace with CUDA events.
+// Autotuner: picks, for the static solver on FP32 cubes up to 128^3, whether the
+// forward half of the CG iteration runs as a plane pass, by timing a chunk of CG
+// iterations (pd_plan_autotune_solve) on the plan's own workspace with CUDA
+// events.
 //
-// The search covers (for the solver on FP32 cubes up to 128^3) whether the CG
-// iteration's forward half runs as a plane pass, then rows x stages jointly, the inverse passes'
-// stages, the schedule, the last-axis width and the x2 width one at a time; each candidate is timed as
-// the median of nine force evaluations after three untimed ones. Candidates
-// are limited to the shapes the passes accept (powers of two; at least one
-// warp per row block; shared memory within the pass's own limit, which the
-// configuration functions enforce by shrinking the candidate). The
-// transforms compute the same values for every candidate (only the order of
-// block partial sums in the solvers' inner products changes).
-#include <algorithm>
+// The tile shapes of the row and column passes are compile-time constants per
+// axis length (pd_rows.cuh, pd_cols.cuh): with the length and the shape known
+// the index arithmetic folds away, which gained more than any choice of shape
+// at run time did. The tuning record (pd_plan_tuning, pd_plan_set_tuning) keeps
+// its six entries; autotuning reports the nominal shape in those that are 0.
 #include <map>
 #include <tuple>
-#include <vector>
 
-#include "pd_force_impl.cuh"
+#include "pd_plan.cuh"
 
 using namespace pd;
 
@@ -30,8 +22,6 @@ extern "C" int pd_batch_size(const pd_batch *B);
 
 namespace pd {
 pd_status time_cg_chunk(pd_plan *p, cudaEvent_t e0, cudaEvent_t e1, float *ms_out);
-template <typename T>
-pd_status force_nl(pd_plan *p, const T *u, T *L, cudaStream_t st);
 }
 
 namespace {
@@ -45,114 +35,48 @@ void drop_graphs(pd_plan *p)
         }
 }
 
-template <typename T>
-pd_status time_force(pd_plan *p, cudaEvent_t e0, cudaEvent_t e1, float *ms_out)
-{
-    cudaStream_t st = p->own_stream;
-    const T *u = (const T *)p->cg_e;
-    T *L = (T *)p->cg_q;
-    auto eval = [&]() { return p->nonlinear ? force_nl<T>(p, u, L, st) : force_plain<T>(p, u, nullptr, L, nullptr, st); };
-    for (int k = 0; k < 3; ++k) PD_TRY(eval());
-    std::vector<float> t;
-    for (int k = 0; k < 9; ++k) {
-        PD_CUDA_TRY(cudaEventRecord(e0, st));
-        PD_TRY(eval());
-        PD_CUDA_TRY(cudaEventRecord(e1, st));
-        PD_CUDA_TRY(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        PD_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-        t.push_back(ms);
-    }
-    std::sort(t.begin(), t.end());
-    *ms_out = t[4];
-    return PD_OK;
-}
-
-// what the search times: 0 a force evaluation, 1 a chunk of static-solver
-// CG iterations (its graph is recaptured for every candidate)
-pd_status time_cfg(pd_plan *p, int target, cudaEvent_t e0, cudaEvent_t e1, float *ms)
-{
-    if (target == 1) {
-        drop_graphs(p);
-        return time_cg_chunk(p, e0, e1, ms);
-    }
-    return p->prob.fp64 ? time_force<double>(p, e0, e1, ms) : time_force<float>(p, e0, e1, ms);
-}
-
+// target 1: the static solver's CG iteration, 0: force evaluations (nothing to choose)
 pd_status tune_plan(pd_plan *p, cudaStream_t caller, int target = 0)
 {
-    PD_CUDA_TRY(cudaEventRecord(p->ev_join[0], caller));
-    PD_CUDA_TRY(cudaStreamWaitEvent(p->own_stream, p->ev_join[0], 0));
-    const size_t bytes = (size_t)p->dim * p->N * (p->prob.fp64 ? 8 : 4);
-    PD_CUDA_TRY(cudaMemsetAsync(p->cg_e, 0, bytes, p->own_stream));
-    const int prof = p->prof_on;
-    p->prof_on = 0;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    PD_CUDA_TRY(cudaEventCreate(&e0));
-    PD_CUDA_TRY(cudaEventCreate(&e1));
-    pd_status s = PD_OK;
-    auto best_of = [&](int *knob, const std::vector<int> &cands) {
-        if (s != PD_OK || cands.size() < 2) return;
-        int best = *knob;
+    // the inverse plane pass is not a candidate: a lone chunk timed it faster,
+    // whole solves slower (128^3: 115.3 against 105.9 ms per solve)
+    if (target == 1 && p->dim == 3 && !p->prob.fp64 && !p->state_based && p->n1 == p->n2 &&
+        (p->n1 == 32 || p->n1 == 64 || p->n1 == 128)) {
+        PD_CUDA_TRY(cudaEventRecord(p->ev_join[0], caller));
+        PD_CUDA_TRY(cudaStreamWaitEvent(p->own_stream, p->ev_join[0], 0));
+        const int prof = p->prof_on;
+        p->prof_on = 0;
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        PD_CUDA_TRY(cudaEventCreate(&e0));
+        PD_CUDA_TRY(cudaEventCreate(&e1));
+        pd_status s = PD_OK;
         float tbest = 1e30f;
-        for (int c : cands) {
-            *knob = c;
+        int best = p->plane_passes;
+        for (int c : {1, 0}) {
+            if (s != PD_OK) break;
+            p->plane_passes = c;
+            drop_graphs(p);
             float ms = 0.f;
-            s = time_cfg(p, target, e0, e1, &ms);
-            if (s != PD_OK) return;
-            if (ms < tbest) {
+            s = time_cg_chunk(p, e0, e1, &ms);
+            if (s == PD_OK && ms < tbest) {
                 tbest = ms;
                 best = c;
             }
         }
-        *knob = best;
-    };
-    // static solve on an FP32 cube with plane passes: whether the forward half
-    // of the CG iteration runs as a plane pass, first, as the row knobs below
-    // only act on the halves that stay row passes. The inverse plane pass is
-    // not a candidate: a lone chunk timed it faster, whole solves slower (128^3:
-    // 115.3 against 105.9 ms per solve).
-    if (target == 1 && p->dim == 3 && !p->prob.fp64 && !p->state_based && p->n1 == p->n2 &&
-        (p->n1 == 32 || p->n1 == 64 || p->n1 == 128))
-        best_of(&p->plane_passes, {1, 0});
-    // rows per tile and pipeline depth jointly (they interact through shared
-    // memory), then the schedule and the column widths one at a time
-    const int H = p->h;
-    const int nt = H >> kLgV;
-    {
-        float tbest = 1e30f;
-        int rbest = p->tune_rows, sbest = p->tune_stages;
-        for (int r = std::max(1, 32 / nt); r * nt <= 256 && s == PD_OK; r *= 2) {
-            if (p->nrows % r) continue;
-            for (int ns : {2, 1}) {
-                p->tune_rows = r;
-                p->tune_stages = ns;
-                float ms = 0.f;
-                s = time_cfg(p, target, e0, e1, &ms);
-                if (s != PD_OK) break;
-                if (ms < tbest) {
-                    tbest = ms;
-                    rbest = r;
-                    sbest = ns;
-                }
-            }
-        }
-        p->tune_rows = rbest;
-        p->tune_stages = sbest;
+        p->plane_passes = best;
+        p->prof_on = prof;
+        drop_graphs(p);
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        if (s != PD_OK) return s;
+        PD_CUDA_TRY(cudaEventRecord(p->ev_join[1], p->own_stream));
+        PD_CUDA_TRY(cudaStreamWaitEvent(caller, p->ev_join[1], 0));
     }
-    best_of(&p->tune_stages_inv, {1, 2});
-    // schedule: only lengths that are not powers of 8 have a remainder stage
-    const bool rem = (ilog2(H) % kLgV) || (ilog2(p->n2) % kLgV) || (p->dim == 3 && (ilog2(p->n3) % kLgV));
-    if (rem) best_of(&p->tune_sched, {0, 1});
-    best_of(&p->tune_w[1], {32, 16, 8, 4});
-    if (p->dim == 3) best_of(&p->tune_w[0], {32, 16, 8, 4});
-    p->prof_on = prof;
-    drop_graphs(p);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (s != PD_OK) return s;
-    PD_CUDA_TRY(cudaEventRecord(p->ev_join[1], p->own_stream));
-    PD_CUDA_TRY(cudaStreamWaitEvent(caller, p->ev_join[1], 0));
+    if (!p->tune_rows) p->tune_rows = row_warp_rows(p->h);
+    for (int k = 0; k < 2; ++k)
+        if (!p->tune_w[k]) p->tune_w[k] = p->prob.fp64 ? 8 : 16;
+    if (!p->tune_stages) p->tune_stages = 1;
+    if (!p->tune_stages_inv) p->tune_stages_inv = 1;
     return PD_OK;
 }
 
