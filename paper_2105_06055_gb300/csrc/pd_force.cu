@@ -1,4 +1,4 @@
-// pd_force entry point; the pipelines are instantiated in pd_force_f32.cu / pd_force_f64.cu.
+// pd_force entry point; the pipelines are instantiated in pd_force_f32_3d.cu / pd_force_f64_3d.cu and their 2D units.
 #include "pd_ops.cuh"
 
 namespace pd {

@@ -304,24 +304,38 @@ pd_status force_public(pd_plan *p, const T *u, const T *s, T *L, T *W, cudaStrea
     return force_bond_pipeline<T, 3, false>(p, u, s, nullptr, nullptr, L, W, st, true);
 }
 
-// Instantiated once per precision, in pd_force_f32.cu and pd_force_f64.cu.
-#define PD_FORCE_INSTANCES(EXTERN, T)                                                                             \
+// Instantiated once: the pipelines of each precision and dimension in
+// pd_force_f32_2d.cu, pd_force_f32_3d.cu, pd_force_f64_2d.cu and
+// pd_force_f64_3d.cu, the dispatch with the 3D ones.
+#define PD_FORCE_PIPELINES(EXTERN, T, D)                                                                          \
+    EXTERN template pd_status force_bond_pipeline<T, D, false>(pd_plan *, const T *, const T *, const uint8_t *,   \
+                                                               const T *, T *, T *, cudaStream_t, bool);           \
+    EXTERN template pd_status force_bond_pipeline<T, D, true>(pd_plan *, const T *, const T *, const uint8_t *,    \
+                                                              const T *, T *, T *, cudaStream_t, bool);            \
+    EXTERN template pd_status launch_comb<T, CombForce<T, D, false>>(pd_plan *, const CombForce<T, D, false> &,    \
+                                                                     cudaStream_t);
+#define PD_FORCE_DISPATCH(EXTERN, T)                                                                              \
     EXTERN template pd_status weight_gfield<T>(pd_plan *, const T *, const uint8_t *, T *, cudaStream_t);          \
     EXTERN template pd_status force_any<T>(pd_plan *, const T *, const T *, const uint8_t *, const T *, T *, T *,  \
                                            cudaStream_t);                                                          \
     EXTERN template pd_status force_plain<T>(pd_plan *, const T *, const T *, T *, T *, cudaStream_t);             \
-    EXTERN template pd_status force_public<T>(pd_plan *, const T *, const T *, T *, T *, cudaStream_t);            \
-    EXTERN template pd_status force_bond_pipeline<T, 2, false>(pd_plan *, const T *, const T *, const uint8_t *,   \
-                                                               const T *, T *, T *, cudaStream_t, bool);           \
-    EXTERN template pd_status launch_comb<T, CombForce<T, 2, false>>(pd_plan *, const CombForce<T, 2, false> &,    \
-                                                                     cudaStream_t);                                \
-    EXTERN template pd_status launch_comb<T, CombForce<T, 3, false>>(pd_plan *, const CombForce<T, 3, false> &,    \
-                                                                     cudaStream_t);
-#ifndef PD_FORCE_UNIT_F32
-PD_FORCE_INSTANCES(extern, float)
+    EXTERN template pd_status force_public<T>(pd_plan *, const T *, const T *, T *, T *, cudaStream_t);
+#ifndef PD_FORCE_UNIT
+#define PD_FORCE_UNIT 0
 #endif
-#ifndef PD_FORCE_UNIT_F64
-PD_FORCE_INSTANCES(extern, double)
+#if PD_FORCE_UNIT != 322
+PD_FORCE_PIPELINES(extern, float, 2)
+#endif
+#if PD_FORCE_UNIT != 323
+PD_FORCE_PIPELINES(extern, float, 3)
+PD_FORCE_DISPATCH(extern, float)
+#endif
+#if PD_FORCE_UNIT != 642
+PD_FORCE_PIPELINES(extern, double, 2)
+#endif
+#if PD_FORCE_UNIT != 643
+PD_FORCE_PIPELINES(extern, double, 3)
+PD_FORCE_DISPATCH(extern, double)
 #endif
 
 }  // namespace pd

@@ -40,6 +40,7 @@ pd_status set_smem_attr(const void *func, size_t smem)
     cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) {
         set_error("cudaFuncSetAttribute(%zu bytes): %s", smem, cudaGetErrorString(e));
+        cudaGetLastError();  // the call is refused; later launches are not
         return PD_ERR_CUDA;
     }
     cur = smem;
@@ -618,7 +619,7 @@ void pd_plan_destroy(pd_plan *p)
 {
     if (!p) return;
     void *ptrs[] = {p->chi, p->chi_om, p->mbits, p->hoff, p->mhat64, p->mhat32, p->ghat64, p->ghat32, p->G64, p->G32,
-                    p->goff, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
+                    p->goff, p->hzt32, p->hzt64, p->hzcol, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
                     p->qt64, p->m3inv64, p->qt32, p->m3inv32, p->tw64, p->tw32, p->spec32, p->spec64,
                     p->work, p->red};
     for (void *q : ptrs)
@@ -953,6 +954,22 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
         p->bytes -= (int64_t)(sizeof(double) * nb);
         p->lam_max = 0;
         for (double v : hm) p->lam_max = std::max(p->lam_max, v);
+    }
+
+    // bond tables of the horizon sums on tiles
+    {
+        const HzTile t = hz_tile(dim, n1, n2, n3, hd);
+        if (t.rc <= kHzReach && t.ncol <= kHzMaxCols) {
+            const size_t nv = hz_table_values(dim, t);
+            PD_TRY(dalloc(p, &p->hzcol, sizeof(int2) * hz_col_entries(t)));
+            PD_TRY(dalloc(p, &p->hzt32, sizeof(float) * nv));
+            PD_TRY(dalloc(p, &p->hzt64, sizeof(double) * nv));
+            PD_CUDA_TRY(cudaMemsetAsync(p->hzt32, 0, sizeof(float) * nv, st));
+            PD_CUDA_TRY(cudaMemsetAsync(p->hzt64, 0, sizeof(double) * nv, st));
+            k_hz_tables<float><<<1, 256, 0, st>>>(t, hd, dim, pr->dx[0], pr->dx[1], pr->dx[2], p->hzt32, p->hzcol);
+            k_hz_tables<double><<<1, 256, 0, st>>>(t, hd, dim, pr->dx[0], pr->dx[1], pr->dx[2], p->hzt64, p->hzcol);
+            PD_LAUNCH_CHECK();
+        }
     }
 
     // boundary fields

@@ -121,6 +121,11 @@ struct pd_plan {
     int64_t fold_sz = 0;
     double *G64 = nullptr;         // ncomp x N
     float *G32 = nullptr;
+    // bond tables of the horizon sums on tiles (pd_horizon.cuh), null when the
+    // horizon is too large for them
+    float *hzt32 = nullptr;
+    double *hzt64 = nullptr;
+    int2 *hzcol = nullptr;
     int *goff = nullptr;           // nrows + 1: boundary-node list offsets per row
     int *gnode = nullptr;          // [ngent] node of each boundary entry (plane-pass cubes only)
     void *gpe = nullptr;           // [3][ngent] FP32 (G p) per boundary entry, written by the CG iteration

@@ -31,27 +31,36 @@ pd_status force_any(pd_plan *p, const T *u, const T *s, const uint8_t *lam, cons
 
 namespace {
 
-// device counters live in the reduction buffer: [0] flips (int64), [1] flag
+// device counters live in the reduction buffer; the change flag of step s is
+// changed[s & 1], cleared by the step before
 struct VerletCounters {
     unsigned long long flips;
-    int changed;
+    int changed[2];
 };
 
+// First kick, drift and integrity update of step s; with `kick` the second kick
+// of the step before comes first (the force L is the same for both), so that a
+// run of steps reads L, b and v once per step.
 // Gamma values at the end of the step: w + t_next w1 (w1 null: w, constant)
 template <typename T>
 __global__ void k_kick_drift(T *u, T *v, uint8_t *lam, const T *L, const T *b, const T *w, const T *w1, T t_next,
                              const T *W, const uint8_t *chi, const uint8_t *co, int d, int64_t N, T hdt_rho, T dt,
-                             T Wc, int breaking, VerletCounters *cnt)
+                             T Wc, int breaking, int kick, int s, VerletCounters *cnt)
 {
     unsigned long long flips = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) cnt->changed[(s + 1) & 1] = 0;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
         for (int i = 0; i < d; ++i) {
             const int64_t q = i * N + p;
-            const T vh = v[q] + hdt_rho * (L[q] + b[q]);
+            const T a = hdt_rho * (L[q] + b[q]);
+            const bool on = co[q] != 0;
+            T vn = v[q];
+            if (kick) vn = on ? vn + a : T(0);
+            const T vh = vn + a;
             v[q] = vh;
             T g = w ? w[q] : T(0);
             if (w1) g = g + t_next * w1[q];
-            u[q] = co[q] ? (u[q] + dt * vh) : g;
+            u[q] = on ? (u[q] + dt * vh) : g;
         }
         if (breaking && chi[p] && lam[p] && !(W[p] <= Wc)) {
             lam[p] = 0;
@@ -62,7 +71,7 @@ __global__ void k_kick_drift(T *u, T *v, uint8_t *lam, const T *L, const T *b, c
     for (int o = 16; o > 0; o >>= 1) flips += __shfl_down_sync(0xffffffffu, flips, o);
     if ((threadIdx.x & 31) == 0 && flips) {
         atomicAdd(&cnt->flips, flips);
-        atomicExch(&cnt->changed, 1);
+        atomicExch(&cnt->changed[s & 1], 1);
     }
 }
 
@@ -72,8 +81,6 @@ __global__ void k_kick(T *v, const T *L, const T *b, const uint8_t *co, int64_t 
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
         v[q] = co[q] ? v[q] + hdt_rho * (L[q] + b[q]) : T(0);
 }
-
-__global__ void k_clear_changed(VerletCounters *cnt) { cnt->changed = 0; }
 
 // W(x) = 1/2 chi lam Σ_H chi' lam' eta.C(xi).eta dV, eta = u(x+xi) - u(x)
 // (Eq. 47 with the integrity weights of Eq. 44; periodic neighbour offsets).
@@ -125,39 +132,70 @@ __global__ void k_energy_direct(int n1, int n2, int n3, HorizonDev hz, double dx
     }
 }
 
-// The same sum on shared-memory tiles (pd_horizon.cuh): the weight mask and u
-// of a tile with its halo are loaded once, the bond table is a few vectors per
-// bond, shared by the thread's kNodes nodes.
+// One column of bonds of the same sum (pd_horizon.cuh). MASK: neighbours whose
+// weight is 0 add nothing; without it the whole tile has weight 1.
+template <typename T, int D, int Z, bool MASK>
+__device__ __forceinline__ void energy_column(const T *tu, const uint8_t *tm, int tile, const T *bond, int e, int step,
+                                              int rc, const T (&up)[kNodes][D], T (&acc)[kNodes])
+{
+    T a[kNodes + 2 * Z][D];
+    bool in[kNodes + 2 * Z];
+#pragma unroll
+    for (int z = 0; z < kNodes + 2 * Z; ++z) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) a[z][j] = tu[j * tile + e + (z - Z) * step];
+        in[z] = !MASK || tm[e + (z - Z) * step];
+    }
+#pragma unroll
+    for (int oc = -Z; oc <= Z; ++oc) {
+        T x[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[j] = bond[4 * (rc + oc) + j];
+        const T w = bond[4 * (rc + oc) + 3];
+#pragma unroll
+        for (int m = 0; m < kNodes; ++m) {
+            T s = T(0);
+#pragma unroll
+            for (int j = 0; j < D; ++j) s += x[j] * (a[m + Z + oc][j] - up[m][j]);
+            const T next = acc[m] + w * s * s;
+            acc[m] = in[m + Z + oc] ? next : acc[m];
+        }
+    }
+}
+
+// The same sum on shared-memory tiles, column by column; the column of the
+// node itself has weight 0 at oc = 0. Tiles entirely of weight 1 (most of a
+// body) take the loop without masks.
 template <typename T, int D>
 __global__ void __launch_bounds__(kHzX *kHzY)
-    k_energy_tile(HzTile t, HorizonDev hz, double dx1, double dx2, double dx3, const uint8_t *__restrict__ chi,
-                  const uint8_t *__restrict__ lam, const T *__restrict__ u, T *__restrict__ W, int64_t N)
+    k_energy_tile(HzTile t, HzTables<T> tab, const uint8_t *__restrict__ chi, const uint8_t *__restrict__ lam,
+                  const T *__restrict__ u, T *__restrict__ W, int64_t N)
 {
-    constexpr int NC = Sym<D>::n;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    T *bond = reinterpret_cast<T *>(sm_raw);             // [cnt][4]: xi, c / |xi|^2
-    int *off = reinterpret_cast<int *>(bond + 4 * hz.cnt);
-    T *tu = reinterpret_cast<T *>(off + ((hz.cnt + 3) & ~3));  // [D][tile], 0 where the weight is 0
+    T *bond = reinterpret_cast<T *>(sm_raw);  // [columns][2 rc + 1][4]: xi, c / |xi|^2
+    const int nz = 2 * t.rc + 1, slots = t.ncol * nz;
+    int2 *col = reinterpret_cast<int2 *>(bond + 4 * slots);
+    T *tu = reinterpret_cast<T *>(col + ((t.ncol + 1) & ~1));  // [D][tile], 0 where the weight is 0
     const int tile = t.p * t.rows * t.nz;
     uint8_t *tm = reinterpret_cast<uint8_t *>(tu + (size_t)D * tile);  // weight mask
     const int tid = threadIdx.y * kHzX + threadIdx.x;
-    for (int c = tid; c < hz.cnt; c += kHzX * kHzY) {
-        const double x[3] = {hz.off[3 * c] * dx1, hz.off[3 * c + 1] * dx2, hz.off[3 * c + 2] * dx3};
-        double tr = 0.0, r2 = 0.0;
-        for (int k = 0; k < NC; ++k)
-            if (Sym<D>::i(k) == Sym<D>::j(k)) tr += hz.c[k * hz.cnt + c];
-        for (int j = 0; j < D; ++j) r2 += x[j] * x[j];
-        for (int j = 0; j < 3; ++j) bond[4 * c + j] = j < D ? (T)x[j] : T(0);
-        bond[4 * c + 3] = (T)(tr / r2);
-        off[c] = (hz.off[3 * c + 2] * t.rows + hz.off[3 * c + 1]) * t.p + hz.off[3 * c];
+    for (int c = tid; c < slots; c += kHzX * kHzY) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) bond[4 * c + k] = tab.bond[4 * c + k];
     }
+    for (int c = tid; c < t.ncol; c += kHzX * kHzY) col[c] = tab.col[t.ncol + c];
+    bool all = true;
     hz_fill(t, [&](int e, int64_t q) {
-        const bool in = chi[q] && lam[q];
+        const bool in = chi[q] != 0 && lam[q] != 0;
+        T x[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[j] = u[j * N + q];
+        all = all && in;
         tm[e] = in ? 1 : 0;
 #pragma unroll
-        for (int j = 0; j < D; ++j) tu[j * tile + e] = in ? u[j * N + q] : T(0);
+        for (int j = 0; j < D; ++j) tu[j * tile + e] = in ? x[j] : T(0);
     });
-    __syncthreads();
+    const bool full = __syncthreads_and(all);
     const int e0 = hz_elem0(t);
     T up[kNodes][D], acc[kNodes];
 #pragma unroll
@@ -166,23 +204,27 @@ __global__ void __launch_bounds__(kHzX *kHzY)
 #pragma unroll
         for (int j = 0; j < D; ++j) up[m][j] = tu[j * tile + e0 + m * t.step];
     }
-#pragma unroll 2
-    for (int c = 0; c < hz.cnt; ++c) {
-        const int d = e0 + off[c];
-        T x[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) x[j] = bond[4 * c + j];
-        const T w = bond[4 * c + 3];
-#pragma unroll
-        for (int m = 0; m < kNodes; ++m) {
-            const int e = d + m * t.step;
-            T s = T(0);
-#pragma unroll
-            for (int j = 0; j < D; ++j) s += x[j] * (tu[j * tile + e] - up[m][j]);
-            const T next = acc[m] + w * s * s;
-            acc[m] = tm[e] ? next : acc[m];
-        }
+    const int *grp = tab.grp + kHzReach + 2;
+#define PD_ENERGY_COLUMNS(Z, MASK)                                                                       \
+    _Pragma("unroll 1") for (int c = __ldg(grp + Z); c < __ldg(grp + Z + 1); ++c)                         \
+    {                                                                                                    \
+        const int2 k = col[c];                                                                           \
+        energy_column<T, D, Z, MASK>(tu, tm, tile, bond + 4 * k.y, e0 + k.x, t.step, t.rc, up, acc);     \
     }
+    if (full) {
+        PD_ENERGY_COLUMNS(0, false)
+        PD_ENERGY_COLUMNS(1, false)
+        PD_ENERGY_COLUMNS(2, false)
+        PD_ENERGY_COLUMNS(3, false)
+        PD_ENERGY_COLUMNS(4, false)
+    } else {
+        PD_ENERGY_COLUMNS(0, true)
+        PD_ENERGY_COLUMNS(1, true)
+        PD_ENERGY_COLUMNS(2, true)
+        PD_ENERGY_COLUMNS(3, true)
+        PD_ENERGY_COLUMNS(4, true)
+    }
+#undef PD_ENERGY_COLUMNS
 #pragma unroll
     for (int m = 0; m < kNodes; ++m) {
         int64_t p;
@@ -196,13 +238,13 @@ pd_status energy_direct(pd_plan *p, const T *u, const uint8_t *lam, T *W, cudaSt
     const int cnt = p->hdev.cnt;
     {
         const HzTile t = hz_tile(p->dim, p->n1, p->n2, p->n3, p->hdev);
-        const size_t ts = (size_t)4 * cnt * sizeof(T) + (size_t)((cnt + 3) & ~3) * sizeof(int) +
+        const size_t ts = (size_t)4 * t.ncol * (2 * t.rc + 1) * sizeof(T) +
+                          (size_t)((t.ncol + 1) & ~1) * sizeof(int2) +
                           (size_t)t.p * t.rows * t.nz * (p->dim * sizeof(T) + 1);
-        if (ts <= kHzSmem) {
+        if (ts <= kHzSmem && t.rc <= kHzReach && p->hzcol) {
             const auto kern = p->dim == 3 ? k_energy_tile<T, 3> : k_energy_tile<T, 2>;
             PD_TRY(set_smem_attr((const void *)kern, ts));
-            kern<<<hz_grid(t), dim3(kHzX, kHzY), ts, st>>>(t, p->hdev, p->prob.dx[0], p->prob.dx[1], p->prob.dx[2],
-                                                           p->chi, lam, u, W, p->N);
+            kern<<<hz_grid(t), dim3(kHzX, kHzY), ts, st>>>(t, hz_tables<T>(p, t), p->chi, lam, u, W, p->N);
             PD_LAUNCH_CHECK();
             p->launches++;
             return PD_OK;
@@ -260,17 +302,17 @@ pd_status verlet_impl(pd_plan *p, T *u, T *v, uint8_t *lam, const T *b, const T 
     for (int s = 0; s < nsteps; ++s) {
         const T t_next = (T)(t0 + (double)(s + 1) * dt);
         k_kick_drift<T><<<ng, 256, 0, st>>>(u, v, lam, L, b, w, w1, t_next, W, p->chi, p->chi_om, d, N, hdt,
-                                            (T)dt, (T)p->wc, breaking, cnt);
+                                            (T)dt, (T)p->wc, breaking, s > 0 ? 1 : 0, s, cnt);
         PD_LAUNCH_CHECK();
         p->launches++;
         if (breaking) {
             // G^lam, skipped unless this step's kick-drift flagged a change
-            PD_TRY((launch_gfield<T, uint8_t>(p, lam, G, &cnt->changed, st)));
-            k_clear_changed<<<1, 1, 0, st>>>(cnt);
-            PD_LAUNCH_CHECK();
-            p->launches += 2;
+            PD_TRY((launch_gfield<T, uint8_t>(p, lam, G, &cnt->changed[s & 1], st)));
+            p->launches++;
         }
         PD_TRY(step_force<T>(p, u, lam, G, L, W, breaking, st));
+    }
+    if (nsteps > 0) {
         k_kick<T><<<ngv, 256, 0, st>>>(v, L, b, p->chi_om, d * N, hdt);
         PD_LAUNCH_CHECK();
         p->launches++;
