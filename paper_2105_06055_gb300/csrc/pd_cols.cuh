@@ -77,7 +77,7 @@ __device__ __forceinline__ void dft_n(cx<T> *v)
 
 // Shape of a pass of length 2^LG over FB fields: chunk radix 2^LGC, largest
 // first-stage radix 2^LGM.
-template <typename T, int LG, int FB, int LGC_, int LGM, int WMIN = 64>
+template <typename T, int LG, int FB, int LGC_, int LGM, int WMIN = 64, int WMAX = 128>
 struct ColShape {
     static constexpr int LGC = LGC_ < LG ? LGC_ : LG;
     static constexpr int REM = LG - LGC;
@@ -93,11 +93,11 @@ struct ColShape {
     static constexpr size_t col_bytes(int pad) { return (size_t)FB * (L + (pad ? L / RC : 0)) * sizeof(cx<T>); }
     // Tile width: 128-byte segments while three blocks of the tile fit on an SM
     // (whole warps at least), then narrower, down to WMIN bytes: 64 for 3D boxes
-    // (512^3, 32-byte segments: 2840 us a pass, 64-byte: 1544), 32 for the
-    // cache-resident 2D grids, where more tiles fill more SMs
+    // (512^3, 32-byte segments: 2840 us a pass, 64-byte: 1544). WMAX and WMIN are
+    // 32 for the cache-resident 2D grids, where more tiles fill more SMs
     static constexpr int width()
     {
-        int w = (int)(128 / sizeof(cx<T>));
+        int w = (int)(WMAX / sizeof(cx<T>));
         while (w * NT * G < 32) w <<= 1;
         while (w * (int)sizeof(cx<T>) > WMIN && (col_bytes(0) * w > 70 * 1024 || w * NT * G > 512)) w >>= 1;
         while (w > 2 && col_bytes(1) * w > 220 * 1024) w >>= 1;
@@ -296,7 +296,7 @@ constexpr int comb_lgc()
 template <typename T, class Op, int LG>
 struct CombShape
     : ColShape<T, LG, (Op::kFin > Op::kFout ? Op::kFin : Op::kFout),
-               comb_lgc<T, (Op::kFin > Op::kFout ? Op::kFin : Op::kFout)>(), 3, Op::kDim == 2 ? 32 : 64> {
+               comb_lgc<T, (Op::kFin > Op::kFout ? Op::kFin : Op::kFout)>(), 3, Op::kDim == 2 ? 32 : 64, Op::kDim == 2 ? 32 : 128> {
 };
 // Resident blocks the register allocation has to allow: 128 registers (FP64:
 // 168) or what shared memory allows. Measured at 256^3: radix-8 first stages
