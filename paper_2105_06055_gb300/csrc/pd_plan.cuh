@@ -328,7 +328,8 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     constexpr int FB = Op::kFin > Op::kFout ? Op::kFin : Op::kFout;
     RowGeom g;
     g.lgh = ilog2(p->h);
-    g.rows = row_tile_rows(p->h, FB);
+    const int lgc = row_lgc(sizeof(T) == 8, Op::kDim, g.lgh);
+    g.rows = row_tile_rows(p->h, lgc, FB);
     bool whole = true;  // the tile size the fixed-length kernels are compiled for
     while (p->nrows % g.rows) {
         g.rows >>= 1;
@@ -338,14 +339,14 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     g.err = p->dev_status;
     g.inject = p->inject;
     const size_t smem =
-        16 + (size_t)Op::kNB * g.rows * p->n1 + (size_t)FB * g.rows * row_pitch(p->h) * sizeof(cx<T>);
+        16 + (size_t)Op::kNB * g.rows * p->n1 + (size_t)FB * g.rows * row_pitch(p->h, lgc) * sizeof(cx<T>);
     int64_t grid = p->nrows / g.rows;
     if (op_reduce<Op>::value) grid = std::min<int64_t>(grid, 8 * (int64_t)p->nsm);
     if (grid_out) *grid_out = (unsigned)grid;
     const auto kern = whole ? rows_kernel<T, Op>(g.lgh) : &k_rows<T, Op>;
     PD_TRY(set_smem_attr((const void *)kern, smem));
     PD_TRY(prof_begin(p, Op::kFin > 0 ? PASS_ROWS_INV : PASS_ROWS_FWD, st));
-    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(FB)), smem, st, g, op,
+    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(FB, lgc)), smem, st, g, op,
                     tw_buf<T>(p)));
     PD_TRY(prof_end(p, st));
     p->launches++;

@@ -6,8 +6,8 @@
 // rest is latency (dependent loads of the node work, exchanges between the
 // transform's stages), so the passes are cut into many small independent
 // pieces. A block takes a few rows (as many as one warp transforms at a time)
-// of all fields. The transforms are warp-wide: NT = H/16 lanes hold a row of H
-// packed values, the lanes of a warp 32/NT rows of one field, and a warp's
+// of all fields. The transforms are warp-wide: NT lanes (H/16 or H/8) hold a row of
+// H packed values, the lanes of a warp 32/NT rows of one field, and a warp's
 // stages exchange through its own rows of shared memory with warp barriers
 // only. One block barrier separates the node work (all lanes over consecutive
 // nodes, all fields of a node in one lane) from the transforms (one field per
@@ -20,7 +20,7 @@
 // ones) made 8 to 16 L1 lookups per instruction, and L1 lookups set the pace of
 // the passes (88% busy at 256^3).
 //
-// Between the stages a row carries one pad element per eight, and the row pitch
+// Between the stages a row carries one pad element per chunk, and the row pitch
 // puts the rows of a warp on different banks, which makes the strided stage
 // accesses and the chunk accesses conflict-free. Spectra lie in natural order at
 // the front of the same row.
@@ -32,34 +32,53 @@
 
 namespace pd {
 
-// Row transform of 2^LG packed values: stages RA (RB) 8, 16 or 32 values a lane.
-template <int LG>
+// Chunk radix (log2) of a row of 2^lg packed values: 8, a lane then holds 16
+// values; 4 (8 values a lane, twice the lanes per row) for FP64 and for the 2D
+// grids up to 256 nodes wide. Both have few warps for the chip otherwise: a
+// 128 x 128 plate in FP64 has 256 row transforms, and a warp's FP64 instructions,
+// 64 clocks each, ran one after the other on 8 of the SMs (23 us a pass).
+__host__ __device__ constexpr int row_lgc(bool fp64, int dim, int lg) { return (fp64 || dim == 2) && lg <= 7 ? 2 : 3; }
+
+// Row transform of 2^LG packed values: stages RA (RB) RC.
+template <int LG, int LGC_>
 struct RowShape {
     static constexpr int H = 1 << LG;
-    static constexpr int LGC = 3, RC = 8;
-    static constexpr int REM = LG - LGC;
-    static constexpr int LGA = REM <= 4 ? REM : (REM + 1) / 2;
+    static constexpr int LGC = LGC_, RC = 1 << LGC;
+    static constexpr int NT = H / (2 * RC) < 32 ? H / (2 * RC) : 32;  // lanes per row
+    static constexpr int V = H / NT;
+    static constexpr int REM = LG - LGC, LGV = LG - (NT == 32 ? 5 : LG - LGC - 1);
+    static constexpr int LGA = REM <= LGV && REM <= 4 ? REM : (REM + 1) / 2;
     static constexpr int LGB = REM - LGA;
     static constexpr int RA = 1 << LGA, RB = 1 << LGB, M = H / RA, K = H / RC;
-    static constexpr int MP = M + M / 8;  // first-stage stride with the pad elements
-    static constexpr int NT = H / 16 < 32 ? H / 16 : 32;  // lanes per row
-    static constexpr int V = H / NT;
-    static constexpr int ROWS = 32 / NT;  // rows of a warp
+    static constexpr int MP = M + M / RC;  // first-stage stride with the pad elements
+    static constexpr int ROWS = 32 / NT;   // rows of a warp
     static constexpr int PAIRS = K / 2 / NT;
-    static_assert(LG >= 4 && LG <= 10 && PAIRS >= 1, "row length");
+    static_assert(LG >= 4 && LG <= 10 && PAIRS >= 1 && RA <= V && RB <= V && M % RC == 0, "row length");
 };
-// pitch of a padded row in shared memory (complex elements)
-// (even: rows start on 16-byte boundaries)
-__host__ __device__ constexpr int row_pitch(int H) { return H + H / 8 + (H >= 256 ? 0 : H == 16 ? 2 : H / 16); }
-__host__ __device__ constexpr int row_warp_rows(int H) { return H / 16 < 32 ? 512 / H : 1; }
-__device__ __forceinline__ int row_at(int e) { return e + (e >> 3); }
-// a tile holds the rows one warp transforms at a time, more of them for one or
-// two fields, and a warp per field and such group up to twelve
-__host__ __device__ constexpr int row_groups(int fields) { return fields == 1 ? 4 : fields == 2 ? 2 : 1; }
-__host__ __device__ constexpr int row_tile_rows(int H, int fields) { return row_warp_rows(H) * row_groups(fields); }
-__host__ __device__ constexpr int row_warps(int fields)
+// pitch of a padded row in shared memory (complex elements; even: rows start on
+// 16-byte boundaries), lanes per row and rows of a warp
+__host__ __device__ constexpr int row_lanes(int H, int lgc) { return (H >> (lgc + 1)) < 32 ? H >> (lgc + 1) : 32; }
+__host__ __device__ constexpr int row_pitch(int H, int lgc)
 {
-    const int tasks = fields * row_groups(fields);
+    const int nt = row_lanes(H, lgc);
+    return H + (H >> lgc) + (nt >= 16 ? 0 : nt == 1 ? 2 : nt);
+}
+__host__ __device__ constexpr int row_warp_rows(int H, int lgc) { return 32 / row_lanes(H, lgc); }
+template <int LGC>
+__device__ __forceinline__ int row_at(int e)
+{
+    return e + (e >> LGC);
+}
+// a tile holds the rows one warp transforms at a time, more of them for one
+// or two fields, and a warp per field and such group up to twelve
+__host__ __device__ constexpr int row_groups(int fields, int lgc) { return fields == 1 ? 4 : fields == 2 && lgc == 3 ? 2 : 1; }
+__host__ __device__ constexpr int row_tile_rows(int H, int lgc, int fields)
+{
+    return row_warp_rows(H, lgc) * row_groups(fields, lgc);
+}
+__host__ __device__ constexpr int row_warps(int fields, int lgc)
+{
+    const int tasks = fields * row_groups(fields, lgc);
     int w = tasks;
     for (int k = 2; w > 12; ++k) w = (tasks + k - 1) / k;
     return w;
@@ -93,15 +112,15 @@ __device__ __forceinline__ void row_stage_b(cx<T> *s, int t, const cx<T> *__rest
 // Forward transform of one packed row in shared memory (so: this lane's row) to
 // the packed half spectrum, in place; all lanes of the warp call, those without
 // a row (grids with fewer rows than a warp holds) with on = false.
-template <typename T, int LG>
+template <typename T, int LG, int LGC>
 __device__ __forceinline__ void row_forward(unsigned so, bool on, int t, const cx<T> *__restrict__ tw)
 {
-    using S = RowShape<LG>;
+    using S = RowShape<LG, LGC>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     cx<T> *s = reinterpret_cast<cx<T> *>(smem_raw + so);
 #pragma unroll
     for (int b = 0; on && b < S::V / S::RA; ++b) {
-        const int j = t + b * S::NT, o = row_at(j);
+        const int j = t + b * S::NT, o = row_at<LGC>(j);
         cx<T> v[S::RA];
 #pragma unroll
         for (int r = 0; r < S::RA; ++r) v[r] = s[o + r * S::MP];
@@ -164,10 +183,10 @@ __device__ __forceinline__ void row_forward(unsigned so, bool on, int t, const c
 
 // Inverse transform of a packed half spectrum in shared memory to the packed
 // row, in place: x[2n] = Re, x[2n+1] = Im (unnormalised).
-template <typename T, int LG>
+template <typename T, int LG, int LGC>
 __device__ __forceinline__ void row_inverse(unsigned so, bool on, int t, const cx<T> *__restrict__ tw)
 {
-    using S = RowShape<LG>;
+    using S = RowShape<LG, LGC>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     cx<T> *s = reinterpret_cast<cx<T> *>(smem_raw + so);
     constexpr int C2 = S::RC / 2;
@@ -225,7 +244,7 @@ __device__ __forceinline__ void row_inverse(unsigned so, bool on, int t, const c
     if (!on) return;
 #pragma unroll
     for (int b = 0; b < S::V / S::RA; ++b) {
-        const int j = t + b * S::NT, o = row_at(j);
+        const int j = t + b * S::NT, o = row_at<LGC>(j);
         cx<T> v[S::RA];
 #pragma unroll
         for (int r = 0; r < S::RA; ++r) v[r] = s[o + r * S::MP];
@@ -263,43 +282,32 @@ struct RowCtx {
 };
 
 // one copy of the transforms for the kernels that read the row length at run time
-template <typename T, int LG>
-__device__ __noinline__ void row_forward_call(unsigned s, bool on, int t, const cx<T> *__restrict__ tw)
+template <typename T, int LG, int LGC, bool INV>
+__device__ __noinline__ void row_call(unsigned s, bool on, int t, const cx<T> *__restrict__ tw)
 {
-    row_forward<T, LG>(s, on, t, tw);
+    if constexpr (INV)
+        row_inverse<T, LG, LGC>(s, on, t, tw);
+    else
+        row_forward<T, LG, LGC>(s, on, t, tw);
 }
-template <typename T, int LG>
-__device__ __noinline__ void row_inverse_call(unsigned s, bool on, int t, const cx<T> *__restrict__ tw)
-{
-    row_inverse<T, LG>(s, on, t, tw);
-}
-template <typename T, int LG, bool INV>
+template <typename T, int DIM, int LG, bool INV>
 __device__ __forceinline__ void row_transform(int lgh, unsigned s, bool on, int t, const cx<T> *__restrict__ tw)
 {
+    constexpr bool D = sizeof(T) == 8;
     if constexpr (LG > 0) {
         if constexpr (INV)
-            row_inverse<T, LG>(s, on, t, tw);
+            row_inverse<T, LG, row_lgc(D, DIM, LG)>(s, on, t, tw);
         else
-            row_forward<T, LG>(s, on, t, tw);
-    } else if constexpr (INV) {
-        switch (lgh) {
-            case 4: row_inverse_call<T, 4>(s, on, t, tw); break;
-            case 5: row_inverse_call<T, 5>(s, on, t, tw); break;
-            case 6: row_inverse_call<T, 6>(s, on, t, tw); break;
-            case 7: row_inverse_call<T, 7>(s, on, t, tw); break;
-            case 8: row_inverse_call<T, 8>(s, on, t, tw); break;
-            case 9: row_inverse_call<T, 9>(s, on, t, tw); break;
-            default: row_inverse_call<T, 10>(s, on, t, tw); break;
-        }
+            row_forward<T, LG, row_lgc(D, DIM, LG)>(s, on, t, tw);
     } else {
         switch (lgh) {
-            case 4: row_forward_call<T, 4>(s, on, t, tw); break;
-            case 5: row_forward_call<T, 5>(s, on, t, tw); break;
-            case 6: row_forward_call<T, 6>(s, on, t, tw); break;
-            case 7: row_forward_call<T, 7>(s, on, t, tw); break;
-            case 8: row_forward_call<T, 8>(s, on, t, tw); break;
-            case 9: row_forward_call<T, 9>(s, on, t, tw); break;
-            default: row_forward_call<T, 10>(s, on, t, tw); break;
+            case 4: row_call<T, 4, row_lgc(D, DIM, 4), INV>(s, on, t, tw); break;
+            case 5: row_call<T, 5, row_lgc(D, DIM, 5), INV>(s, on, t, tw); break;
+            case 6: row_call<T, 6, row_lgc(D, DIM, 6), INV>(s, on, t, tw); break;
+            case 7: row_call<T, 7, row_lgc(D, DIM, 7), INV>(s, on, t, tw); break;
+            case 8: row_call<T, 8, row_lgc(D, DIM, 8), INV>(s, on, t, tw); break;
+            case 9: row_call<T, 9, row_lgc(D, DIM, 9), INV>(s, on, t, tw); break;
+            default: row_call<T, 10, row_lgc(D, DIM, 10), INV>(s, on, t, tw); break;
         }
     }
 }
@@ -361,18 +369,20 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int FI = Op::kFin, FO = Op::kFout, NB = Op::kNB, FB = FI > FO ? FI : FO;
     const int lgh = LG > 0 ? LG : g.lgh;
-    const int H = 1 << lgh, n1 = 2 * H, pitch = row_pitch(H);
-    const int rows = LG > 0 ? row_tile_rows(H, FB) : g.rows;
+    const int lgc = row_lgc(sizeof(T) == 8, Op::kDim, lgh);
+    const int H = 1 << lgh, n1 = 2 * H, pitch = row_pitch(H, lgc);
+    const int rows = LG > 0 ? row_tile_rows(H, lgc, FB) : g.rows;
     unsigned long long *mbar = reinterpret_cast<unsigned long long *>(smem_raw);
     uint8_t *nb = smem_raw + 16;
     const unsigned spec_off = 16u + (unsigned)(NB * rows * n1);
     cx<T> *spec = reinterpret_cast<cx<T> *>(smem_raw + spec_off);
     const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
-    const int nt = H / 16 < 32 ? H / 16 : 32, wr = 32 / nt;  // lanes of a row, rows of a warp
+    const int nt = row_lanes(H, lgc), wr = 32 / nt;  // lanes of a row, rows of a warp
+    auto at = [&](int e) { return e + (e >> lgc); };
     const int fstr = rows * pitch;  // field stride of the tile
     // node pairs loaded ahead: about 36 registers' worth
     constexpr int U0 = (int)(144 / sizeof(typename Op::Nd)), U = U0 < 1 ? 1 : U0 > 6 ? 6 : U0;
-    const int lr = lane / nt, lt = lane & (nt - 1), groups = LG > 0 ? row_groups(FB) : rows > wr ? rows / wr : 1;
+    const int lr = lane / nt, lt = lane & (nt - 1), groups = LG > 0 ? row_groups(FB, lgc) : rows > wr ? rows / wr : 1;
     const int64_t ntiles = g.nrows / rows;
     constexpr bool kLoad = FI > 0 || NB > 0;
     if (kLoad && tid == 0) mbar_init(mbar, 1);
@@ -418,7 +428,7 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
                 const int f = task / groups, r = (task - f * groups) * wr + lr;
                 const unsigned s = spec_off + (unsigned)((f * rows + r) * pitch) * (unsigned)sizeof(cx<T>);
                 const bool on = r < rows;
-                row_transform<T, LG, true>(lgh, s, LG > 0 || on, lt, tw);
+                row_transform<T, Op::kDim, LG, true>(lgh, s, LG > 0 || on, lt, tw);
             }
             __syncthreads();
         }
@@ -433,13 +443,13 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
                     const int nd = (int)(p - row0 * n1), rl = nd >> (lgh + 1), i1 = nd & (n1 - 1);
 #pragma unroll
                     for (int f = 0; f < FI; ++f)
-                        base[2 * ((f * rows + rl) * pitch + row_at(i1 >> 1)) + (i1 & 1)] += s[f];
+                        base[2 * ((f * rows + rl) * pitch + at(i1 >> 1)) + (i1 & 1)] += s[f];
                 }
                 __syncthreads();
             }
         }
         const RowCtx ctx{row0, row0 * n1, rows * n1, nb};
-        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(FB) : (int)blockDim.x;
+        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(FB, lgc) : (int)blockDim.x;
         typename Op::Nd nd[U];
         auto load = [&](int i0) {
 #pragma unroll
@@ -458,7 +468,7 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
             for (int u = 0; u < U; ++u) {
                 const int idx = i0 + u * nthr;
                 if (idx < pairs) {
-                    cx<T> *sp = spec + (idx >> lgh) * pitch + row_at(idx & (H - 1));
+                    cx<T> *sp = spec + (idx >> lgh) * pitch + at(idx & (H - 1));
                     T in0[FI > 0 ? FI : 1], in1[FI > 0 ? FI : 1], o0[FO > 0 ? FO : 1], o1[FO > 0 ? FO : 1];
 #pragma unroll
                     for (int f = 0; f < FI; ++f) {
@@ -479,7 +489,7 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
                 const int f = task / groups, r = (task - f * groups) * wr + lr;
                 const unsigned s = spec_off + (unsigned)((f * rows + r) * pitch) * (unsigned)sizeof(cx<T>);
                 const bool on = r < rows;
-                row_transform<T, LG, false>(lgh, s, LG > 0 || on, lt, tw);
+                row_transform<T, Op::kDim, LG, false>(lgh, s, LG > 0 || on, lt, tw);
                 fence_proxy_async();
                 __syncwarp();
                 if (lt == 0 && on) {

@@ -72,7 +72,7 @@ pd_status tune_plan(pd_plan *p, cudaStream_t caller, int target = 0)
         PD_CUDA_TRY(cudaEventRecord(p->ev_join[1], p->own_stream));
         PD_CUDA_TRY(cudaStreamWaitEvent(caller, p->ev_join[1], 0));
     }
-    if (!p->tune_rows) p->tune_rows = row_warp_rows(p->h);
+    if (!p->tune_rows) p->tune_rows = row_warp_rows(p->h, row_lgc(p->prob.fp64 != 0, p->dim, ilog2(p->h)));
     for (int k = 0; k < 2; ++k)
         if (!p->tune_w[k]) p->tune_w[k] = p->prob.fp64 ? 8 : 16;
     if (!p->tune_stages) p->tune_stages = 1;
