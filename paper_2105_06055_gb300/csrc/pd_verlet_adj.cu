@@ -125,12 +125,15 @@ __global__ void k_adj_loss(const T *u, const T *ut, const uint8_t *co, T *ubar, 
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
-// v~ = chi_O (v~ + dt u~)
+// v~ = chi_O (v~ + dt u~) ; y = k v~ (the cotangent of the adjoint force application)
 template <typename T>
-__global__ void k_adj_vbar(T *vbar, const T *ubar, const uint8_t *co, int64_t n, T dt)
+__global__ void k_adj_vbar(T *vbar, const T *ubar, T *y, const uint8_t *co, int64_t n, T dt, T k)
 {
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-        vbar[q] = co[q] ? vbar[q] + dt * ubar[q] : T(0);
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+        const T w = co[q] ? vbar[q] + dt * ubar[q] : T(0);
+        vbar[q] = w;
+        y[q] = k * w;
+    }
 }
 
 // u~ = chi_O (u~ + g_u) ; s~ += g_s lam  (g_u, g_s already for the cotangent k v~)
@@ -145,14 +148,6 @@ __global__ void k_adj_acc(T *ubar, const T *gu, T *sbar, const T *gs, const uint
         }
         if (lam[p]) sbar[p] += gs[p];
     }
-}
-
-// x = k x (the cotangent of the adjoint force application)
-template <typename T>
-__global__ void k_adj_scale(const T *x, T *y, int64_t n, T k)
-{
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-        y[q] = k * x[q];
 }
 
 // dJ/dc_rel = s~ / (2 s)
@@ -212,6 +207,7 @@ struct AdjRun {
     AdjCounters *cnt;
     T h, dt;
     int breaking;
+    bool weighted = false;  // seff and G made
     unsigned ng, ngv;
 
     T *ck_u(int k) const { return (T *)(w + lay.ck_u) + (size_t)k * p->dim * p->N; }
@@ -222,8 +218,11 @@ struct AdjRun {
 
     // s_eff and its boundary field for the current lam (G recomputed when flagged
     // or when force_g), then L (and W when breaking) at u
+    // (without breaking lam, and so both, stay what the first call made them)
     pd_status force(const T *uu, bool force_g)
     {
+        if (!breaking && weighted) return force_any<T>(p, uu, seff, nullptr, G, L, nullptr, st);
+        weighted = true;
         k_adj_weight<T><<<ng, 256, 0, st>>>(s, lam, seff, p->N);
         if (force_g) k_adj_flag<<<1, 1, 0, st>>>(cnt, 1);
         PD_TRY((launch_gfield<T, T>(p, seff, G, &cnt->changed, st)));
@@ -353,11 +352,10 @@ pd_status loss_grad_impl(pd_plan *p, const T *c_rel, const uint8_t *lam0, const 
             if (n + 1 < k1) PD_TRY(R.step(n));
         }
         for (int n = k1 - 1; n >= k0; --n) {
-            k_adj_vbar<T><<<R.ngv, 256, 0, st>>>(R.vbar, R.ubar, p->chi_om, dN, R.dt);
             const T kf = n == 0 ? R.h : T(2) * R.h;
-            k_adj_scale<T><<<R.ngv, 256, 0, st>>>(R.vbar, R.v, dN, kf);  // R.v: the cotangent k v~
+            k_adj_vbar<T><<<R.ngv, 256, 0, st>>>(R.vbar, R.ubar, R.v, p->chi_om, dN, R.dt, kf);  // R.v: k v~
             PD_LAUNCH_CHECK();
-            p->launches += 2;
+            p->launches++;
             // weight and boundary field of lam^n (without breaking lam never
             // changes: the ones of the recomputed segment are current)
             if (R.breaking) {
