@@ -452,11 +452,11 @@ pd_status pd_plan_set_affine_split(pd_plan *plan, int on);
  * (pd_plan_profile kinds 4 and 5) and the spectra make no round trip between
  * them; a clear bit runs that half as a row pass and a column pass along x2
  * (kinds 0, 1, 3), as on every other shape. Same operator either way (the
- * transforms and epilogues do the same arithmetic). Default 1: on the 128^3
- * cube with cavity the forward plane pass makes the solve faster than its row
- * and column passes, while adding the inverse plane pass makes it slower
- * (115.3 against 105.9 ms per solve); pd_plan_autotune_solve times 1 and 0
- * and keeps the faster. PD_ERR_ARG for a null plan or a mask outside 0..3.
+ * transforms and epilogues do the same arithmetic). Default: 1 on planes of
+ * 32 x 32 nodes (32^3: 32.1 us an iteration against 34.5 with row and column
+ * passes), 0 on larger ones (64^3: 38.3 against 41.4 us with mask 1, 128^3:
+ * 108 against 122); pd_plan_autotune_solve times 1 and 0 and keeps the faster.
+ * PD_ERR_ARG for a null plan or a mask outside 0..3.
  */
 pd_status pd_plan_set_plane_passes(pd_plan *plan, int mask);
 

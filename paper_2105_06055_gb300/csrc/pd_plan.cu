@@ -1008,6 +1008,7 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
             PD_TRY(dalloc(p, &p->gpe, sizeof(float) * 3 * (size_t)ng));
             k_gnode<<<nblk(ng, 256), 256, 0, st>>>((const GEntry<float> *)p->gent32, acc, p->gnode);
             PD_LAUNCH_CHECK();
+            p->plane_passes = n1 == 32 ? 1 : 0;
         }
         PD_CUDA_TRY(cudaStreamSynchronize(st));
     }

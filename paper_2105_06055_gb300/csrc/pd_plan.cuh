@@ -188,8 +188,11 @@ struct pd_plan {
     cudaEvent_t ev_fork[2] = {nullptr, nullptr};
     int no_fork = 0;  // set while capturing into conditional-node bodies (single stream there)
     int pdl = 1;      // pass kernels launched as programmatic dependents (griddepcontrol)
-    int plane_passes = 1;  // FP32 CG on cubes up to 128^3: halves of the iteration whose x1 and x2
-                           // transforms run fused in plane passes (bit 0 forward, bit 1 inverse)
+    // FP32 CG on cubes up to 128^3: halves of the iteration whose x1 and x2 transforms
+    // run fused in plane passes (bit 0 forward, bit 1 inverse). By itself 1 on 32-node
+    // planes (32^3: 32.1 us an iteration against 34.5 with row and column passes), 0 on
+    // the larger ones (64^3: 38.3 against 41.4, 128^3: 108 against 122).
+    int plane_passes = 0;
     double prof_ms[kKinds] = {};
     // tuning record (pd_plan_tuning; the passes' shapes are constants per length)
     int tune_rows = 0;
