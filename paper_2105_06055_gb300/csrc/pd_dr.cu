@@ -299,6 +299,7 @@ template <typename T, int D>
 struct EpiDR {
     static constexpr int kFin = D, kFout = 0, kNB = 1, kDim = D;
     static constexpr bool kReduce = true, kEntries = true;
+    static constexpr int kPre = 3 * D;
     using Acc = DrAcc;
     const T *e, *v, *rhs;
     T *F;
@@ -313,6 +314,10 @@ struct EpiDR {
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return bits; }
+    __device__ const T *pre(int k) const
+    {
+        return k < D ? e + k * N : k < 2 * D ? rhs + (k - D) * N : F + (k - 2 * D) * N;
+    }
     __device__ __forceinline__ const int *rows_off() const { return goff; }
     __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {

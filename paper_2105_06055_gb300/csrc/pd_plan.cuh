@@ -323,7 +323,8 @@ auto rows_kernel(int lgh)
 
 // Row pass: tile and warps by row_tile_rows and row_warps (fewer rows when the
 // grid has fewer). Passes with block reductions run on at most 8 blocks per SM
-// (each block writes partial sums), the others on a block per tile. *grid_out
+// (each block writes partial sums), all with as many tiles as far as it goes; the
+// others on a block per tile. *grid_out
 // receives the block count.
 template <typename T, class Op>
 pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_out = nullptr)
@@ -344,7 +345,10 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     const size_t smem =
         16 + (size_t)Op::kNB * g.rows * p->n1 + (size_t)FB * g.rows * row_pitch(p->h, lgc) * sizeof(cx<T>);
     int64_t grid = p->nrows / g.rows;
-    if (op_reduce<Op>::value) grid = std::min<int64_t>(grid, 8 * (int64_t)p->nsm);
+    if (op_reduce<Op>::value) {
+        const int64_t per = (grid + 8 * (int64_t)p->nsm - 1) / (8 * (int64_t)p->nsm);  // tiles a block
+        grid = (grid + per - 1) / per;
+    }
     if (grid_out) *grid_out = (unsigned)grid;
     const auto kern = whole ? rows_kernel<T, Op>(g.lgh) : &k_rows<T, Op>;
     PD_TRY(set_smem_attr((const void *)kern, smem));

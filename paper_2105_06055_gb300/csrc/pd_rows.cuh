@@ -339,6 +339,17 @@ template <class Op>
 struct op_entries<Op, std::void_t<decltype(Op::kEntries)>> : std::bool_constant<Op::kEntries> {
 };
 
+// Ops that read fields of the plan's own (aligned) buffers after their inverse
+// transforms name them for a prefetch to L2: kPre fields, pre(k). The CG's inverse
+// pass reads p and r from memory, one tile at a time, with 17 warps on an SM to
+// cover it (128^3 solve: 184 -> 182 ms).
+template <class Op, class = void>
+struct op_pre : std::integral_constant<int, 0> {
+};
+template <class Op>
+struct op_pre<Op, std::void_t<decltype(Op::kPre)>> : std::integral_constant<int, Op::kPre> {
+};
+
 // Op interface:
 //   static constexpr int kFin, kFout;  packed spectra read (inverse) / written (forward)
 //   static constexpr int kNB;          byte fields bulk-copied for the tile's rows
@@ -363,8 +374,26 @@ struct op_entries<Op, std::void_t<decltype(Op::kEntries)>> : std::bool_constant<
 // LG > 0: compiled for rows of 2^LG packed values (and the tile size launch_rows
 // gives them): index arithmetic then is constants.
 constexpr int kRowThreads = 384;
+// Threads of a block and resident blocks the register allocation has to allow.
+// Rows of up to 128 packed values: 64 registers a thread (FP64: 128); more warps
+// then cover the copies (state-based 256 x 128 x 128: 254 -> 232 us, force at
+// 256^3: 548 -> 538). Ops with reductions, whose accumulators spill then
+// (128^3 solve: 184 -> 209 ms), and longer rows (1024 x 512 fracture steps: 1268 ->
+// 1309 us) keep 80.
+template <typename T, class Op, int LG>
+constexpr int row_threads()
+{
+    return LG > 0 ? 32 * row_warps(Op::kFin > Op::kFout ? Op::kFin : Op::kFout, row_lgc(sizeof(T) == 8, Op::kDim, LG))
+                  : kRowThreads;
+}
+template <typename T, class Op, int LG>
+constexpr int row_blocks()
+{
+    if (LG == 0 || LG > 7 || op_reduce<Op>::value) return (sizeof(T) == 4 ? 768 : 384) / row_threads<T, Op, LG>();
+    return (sizeof(T) == 4 ? 1024 : 512) / row_threads<T, Op, LG>();
+}
 template <typename T, class Op, int LG = 0>
-__global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(RowGeom g, Op op, const cx<T> *__restrict__ tw)
+__global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG>()) k_rows(RowGeom g, Op op, const cx<T> *__restrict__ tw)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int FI = Op::kFin, FO = Op::kFout, NB = Op::kNB, FB = FI > FO ? FI : FO;
@@ -415,6 +444,15 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
                 }
             }
         }
+        if constexpr (op_pre<Op>::value > 0) {
+            if (tid < op_pre<Op>::value)
+                bulk_prefetch_l2(op.pre(tid) + row0 * n1, (unsigned)(rows * n1 * (int)sizeof(T)));
+        }
+        int k0 = 0, k1 = 0;
+        if constexpr (op_entries<Op>::value) {
+            k0 = op.rows_off()[row0];
+            k1 = op.rows_off()[row0 + rows];
+        }
         // false: the wait ran out (no copy is in flight then: the stalled block issued none)
         auto arrive = [&]() {
             const bool ok = mbar_wait(mbar, phase, g.err);
@@ -433,7 +471,6 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) k_rows(Ro
             __syncthreads();
         }
         if constexpr (op_entries<Op>::value) {
-            const int k0 = op.rows_off()[row0], k1 = op.rows_off()[row0 + rows];
             if (k1 > k0) {
                 T *base = reinterpret_cast<T *>(spec);
                 for (int k = k0 + tid; k < k1; k += blockDim.x) {

@@ -207,6 +207,7 @@ struct EpiCG {
     static constexpr int kFin = D, kFout = 0, kNB = 1, kDim = D;
     static constexpr bool kReduce = true, kEntries = true;
     using Acc = CgAcc;
+    static constexpr int kPre = 2 * D;
     const T *pv, *r;
     const uint8_t *bits;
     const GEntry<T> *gent;
@@ -220,6 +221,7 @@ struct EpiCG {
     __device__ const cx<T> *spec_in(int f) const { return spec + f * fstride; }
     __device__ cx<T> *spec_out(int) const { return nullptr; }
     __device__ const uint8_t *nb_src(int) const { return bits; }
+    __device__ const T *pre(int k) const { return k < D ? pv + k * N : r + (k - D) * N; }
     __device__ __forceinline__ const int *rows_off() const { return goff; }
     __device__ __forceinline__ void entry(int k, int64_t &p, T *s) const
     {
