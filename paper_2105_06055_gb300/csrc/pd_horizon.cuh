@@ -68,7 +68,7 @@ __device__ __forceinline__ void hz_fill(const HzTile &t, Fill fill)
 {
     const int x0 = blockIdx.x * kHzX - t.r1, y0 = blockIdx.y * (t.two ? kHzY * kNodes : kHzY) - t.r2;
     const int z0 = t.two ? 0 : (int)blockIdx.z * kNodes - t.r3;
-    // one warp per row of the tile, two columns of 32 and a remainder per lane;
+    // one warp per row of the tile, two columns per lane (more past 64);
     // (y, z) run along without divisions
     const int lane = threadIdx.x;
     int yr = threadIdx.y, zr = 0;
@@ -76,19 +76,27 @@ __device__ __forceinline__ void hz_fill(const HzTile &t, Fill fill)
         yr -= t.rows;
         ++zr;
     }
-#pragma unroll 2
+    const bool rest = lane + 32 < t.p;
+    const int xa = (x0 + lane) & (t.n1 - 1), xb = (x0 + lane + 32) & (t.n1 - 1);
+#pragma unroll 4
     while (zr < t.nz) {
         const int y = (y0 + yr) & (t.n2 - 1), z = t.two ? 0 : (z0 + zr) & (t.n3 - 1);
         const int64_t row = ((int64_t)z * t.n2 + y) * t.n1;
-        const int e = (zr * t.rows + yr) * t.p;
-        fill(e + lane, row + ((x0 + lane) & (t.n1 - 1)));
-        for (int x = lane + 32; x < t.p; x += 32) fill(e + x, row + ((x0 + x) & (t.n1 - 1)));
+        const int e = (zr * t.rows + yr) * t.p + lane;
+        fill(e, row + xa);
+        if (rest) fill(e + 32, row + xb);
         yr += kHzY;
         while (yr >= t.rows) {
             yr -= t.rows;
             ++zr;
         }
     }
+    if (t.p > 64)  // reach above 16 cells (uneven spacings)
+        for (int r = threadIdx.y; r < t.rows * t.nz; r += kHzY) {
+            const int y = (y0 + r % t.rows) & (t.n2 - 1), z = t.two ? 0 : (z0 + r / t.rows) & (t.n3 - 1);
+            const int64_t row = ((int64_t)z * t.n2 + y) * t.n1;
+            for (int x = lane + 64; x < t.p; x += 32) fill(r * t.p + x, row + ((x0 + x) & (t.n1 - 1)));
+        }
 }
 
 // Tile element and node of this thread's node m; false past the grid (2D, n2 < 32).
@@ -226,7 +234,11 @@ __device__ __forceinline__ void gfield_column(const T *tile, const T *coef, int 
     for (int oc = CENTER ? 1 : -Z; oc <= Z; ++oc) {
         T w[NC];
 #pragma unroll
-        for (int k = 0; k < NC; ++k) w[k] = coef[CP * (rc + oc) + k];
+        for (int k = 0; k < NC; k += 2) {  // CP is even, the table on a 16-byte boundary
+            const typename vec2<T>::type c2 = *reinterpret_cast<const typename vec2<T>::type *>(coef + CP * (rc + oc) + k);
+            w[k] = c2.x;
+            if (k + 1 < NC) w[k + 1] = c2.y;
+        }
 #pragma unroll
         for (int m = 0; m < kNodes; ++m) {
             const T dv = (a[m + Z + oc] - v[m]) + (b[m + Z - oc] - v[m]);
@@ -236,9 +248,13 @@ __device__ __forceinline__ void gfield_column(const T *tile, const T *coef, int 
     }
 }
 
-// The same field on tiles, column by column.
+// The same field on tiles, column by column. Bound by instruction issue (the sums
+// are half of its instructions, the rest loads and the fill of the halo tile) and,
+// below four blocks an SM, by the latency of the fill: 111 us at 128^3 and 122 bonds
+// with 80 registers and rows filled two at a time, 97 with 64 registers and four.
+// 8 nodes per thread issue 12% fewer instructions but need 128 registers: 113 us.
 template <typename T, typename V, int NC>
-__global__ void __launch_bounds__(kHzX *kHzY) k_gfield_tile(HzTile t, HzTables<T> tab,
+__global__ void __launch_bounds__(kHzX *kHzY, sizeof(T) == 4 ? 4 : 1) k_gfield_tile(HzTile t, HzTables<T> tab,
                                                            const uint8_t *__restrict__ chi,
                                                            const V *__restrict__ s, T *__restrict__ G, int64_t N,
                                                            const int *changed)

@@ -1,6 +1,6 @@
 """The horizon sums on shared-memory tiles (boundary field of a node weight,
 Eq. 47 energy density) at the edges of their tiles: a 2D grid lower than one
-tile, the smallest 3D box, tiles that wrap around the box, and a horizon whose
+tile, the smallest 3D box, tiles that wrap around the box, a reach of 20 cells, and a horizon whose
 tile does not fit (the sums that read global memory), against the oracle.
 
 Tolerances are those of the force tests: 1e-11 relative L2 in FP64 (rounding
@@ -72,3 +72,23 @@ def test_breaking_by_the_energy_sum(pdm, oracle, shape, delta):
     plan.close()
     assert np.array_equal(ld.cpu().numpy(), lo)
     assert np.linalg.norm(ud.cpu().numpy() - uo) / np.linalg.norm(uo) < 1e-11
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("shape,dx,delta", [((32, 128), (0.1, 1.0), 2.0), ((16, 16, 64), (0.1, 1.0, 1.0), 2.0)])
+def test_long_reach_along_x1(pdm, oracle, shape, dx, delta, fp64):
+    """A horizon of 20 cells along x1 (uneven spacings): rows of the tile longer than two columns per lane."""
+    g = inputs.rng(7)
+    d = len(shape)
+    chi = np.zeros(shape, np.uint8)
+    chi[(slice(2, -2),) * (d - 1) + (slice(20, -20),)] = 1
+    chi[g.random(shape) < 0.1] = 0
+    dt = torch.float64 if fp64 else torch.float32
+    u = torch.tensor(g.normal(size=(d,) + shape), dtype=dt, device=DEV)
+    s = torch.tensor(0.5 + g.random(shape), dtype=dt, device=DEV)
+    plan = pdm.Plan(pdm.Problem(shape=shape, dx=dx, delta=delta, fp64=fp64), torch.tensor(chi, device=DEV))
+    L = plan.force(u, s=s).double().cpu().numpy()
+    plan.close()
+    ref = oracle.force_bond(u.double().cpu().numpy(), chi, dx, delta, oracle.alpha_bond(d, 1.0, delta),
+                            s=s.double().cpu().numpy())
+    assert np.linalg.norm(L - ref) / np.linalg.norm(ref) < (1e-11 if fp64 else 1e-5)
