@@ -90,7 +90,8 @@ struct ColShape {
     // Field groups: with many fields the stages run on separate fields in
     // parallel (each group takes every G-th field) and the chunks are shared out
     static constexpr int G = FB >= 12 && V / RC >= 8 ? 8 : FB >= 5 && V / RC >= 4 ? 4 : FB >= 5 && V / RC >= 2 ? 2 : 1;
-    static constexpr size_t col_bytes(int pad) { return (size_t)FB * (L + (pad ? L / RC : 0)) * sizeof(cx<T>); }
+    static constexpr int LGP = LGC < 3 ? 3 : LGC;  // rows per pad row
+    static constexpr size_t col_bytes(int pad) { return (size_t)FB * (L + (pad ? L >> LGP : 0)) * sizeof(cx<T>); }
     // Tile width: 128-byte segments while three blocks of the tile fit on an SM
     // (whole warps at least), then narrower, down to WMIN bytes: 64 for 3D boxes
     // (512^3, 32-byte segments: 2840 us a pass, 64-byte: 1544). WMAX and WMIN are
@@ -106,13 +107,14 @@ struct ColShape {
     static constexpr int W = width();
     static constexpr int LGW = W == 16 ? 4 : W == 8 ? 3 : W == 4 ? 2 : 1;
     // rows narrower than the 32 banks: one pad row per chunk keeps the chunk
-    // accesses of neighbouring lanes on different banks
+    // accesses of neighbouring lanes on different banks (chunks of 4: one per two
+    // chunks, so that two blocks of the 12-field pass fit on an SM)
     static constexpr bool PAD = W * sizeof(cx<T>) < 128 && RC >= 4;
     static constexpr int THREADS = W * NT * G;
-    static constexpr int FSZ = (L + (PAD ? L / RC : 0)) * W;  // field stride in shared memory
+    static constexpr int FSZ = (L + (PAD ? L >> LGP : 0)) * W;  // field stride in shared memory
     static constexpr size_t smem = (size_t)FB * FSZ * sizeof(cx<T>);
     static_assert(W * NT * G >= 32, "whole warps");
-    __device__ static __forceinline__ int at(int loc, int c) { return ((PAD ? loc + (loc >> LGC) : loc) << LGW) + c; }
+    __device__ static __forceinline__ int at(int loc, int c) { return ((PAD ? loc + (loc >> LGP) : loc) << LGW) + c; }
 };
 
 template <typename T>
