@@ -208,7 +208,8 @@ __global__ void k_dr_ir_update(double *u, const T *e, const uint8_t *co, int64_t
 __global__ void __launch_bounds__(kFinishThreads) k_dr_finish(double *red, int nparts)
 {
     double a = 0.0, b = 0.0, f = 0.0, z = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nparts; i += kFinishThreads) {
         a += red[kRedPart + 3 * i];
         b += red[kRedPart + 3 * i + 1];
         f += red[kRedPart + 3 * i + 2];

@@ -329,6 +329,24 @@ __global__ void k_gfill(int n1, int64_t nrows, const uint8_t *chi, const double 
     }
 }
 
+// Twiddle tables of every length 2^k <= 2^lgl and radix from the plain table of
+// 2^lgl, which is in its place in tw64 (layout: tw_base)
+__global__ void k_twiddles(int lgl, cx<double> *tw64, cx<float> *tw32)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= tw_entries(lgl)) return;
+    const cx<double> *plain = tw64 + tw_base(lgl, 0);
+    const int k = 31 - __clz(t / kTwRadices + 1), o = t - kTwRadices * ((1 << k) - 1);
+    const int r = o >> k, i = o & ((1 << k) - 1);
+    cx<double> w = mk(1.0, 0.0);
+    if (r <= k) {
+        const int e = r ? (i >> r) * (i & ((1 << r) - 1)) : i;  // j q at j 2^r + q
+        w = plain[e << (lgl - k)];
+    }
+    if (k < lgl || r > 0) tw64[t] = w;
+    tw32[t] = mk((float)w.x, (float)w.y);
+}
+
 // gnode[e] = node of boundary entry e
 __global__ void k_gnode(const GEntry<float> *g, int64_t n, int *gnode)
 {
@@ -619,7 +637,7 @@ void pd_plan_destroy(pd_plan *p)
 {
     if (!p) return;
     void *ptrs[] = {p->chi, p->chi_om, p->mbits, p->hoff, p->mhat64, p->mhat32, p->ghat64, p->ghat32, p->G64, p->G32,
-                    p->goff, p->hzt32, p->hzt64, p->hzcol, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
+                    p->goff, p->hzt64, p->gnode, p->gpe, p->gent64, p->gent32, p->aff_tab, p->aff_coef, p->chat64, p->chat32, p->nlb,
                     p->qt64, p->m3inv64, p->qt32, p->m3inv32, p->tw64, p->tw32, p->spec32, p->spec64,
                     p->work, p->red};
     for (void *q : ptrs)
@@ -961,11 +979,11 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
         const HzTile t = hz_tile(dim, n1, n2, n3, hd);
         if (t.rc <= kHzReach && t.ncol <= kHzMaxCols) {
             const size_t nv = hz_table_values(dim, t);
-            PD_TRY(dalloc(p, &p->hzcol, sizeof(int2) * hz_col_entries(t)));
-            PD_TRY(dalloc(p, &p->hzt32, sizeof(float) * nv));
-            PD_TRY(dalloc(p, &p->hzt64, sizeof(double) * nv));
-            PD_CUDA_TRY(cudaMemsetAsync(p->hzt32, 0, sizeof(float) * nv, st));
-            PD_CUDA_TRY(cudaMemsetAsync(p->hzt64, 0, sizeof(double) * nv, st));
+            // one block: the FP64 values, the FP32 values, the columns
+            PD_TRY(dalloc(p, &p->hzt64, (sizeof(double) + sizeof(float)) * nv + sizeof(int2) * hz_col_entries(t)));
+            p->hzt32 = reinterpret_cast<float *>(p->hzt64 + nv);
+            p->hzcol = reinterpret_cast<int2 *>(p->hzt32 + nv);
+            PD_CUDA_TRY(cudaMemsetAsync(p->hzt64, 0, (sizeof(double) + sizeof(float)) * nv, st));
             k_hz_tables<float><<<1, 256, 0, st>>>(t, hd, dim, pr->dx[0], pr->dx[1], pr->dx[2], p->hzt32, p->hzcol);
             k_hz_tables<double><<<1, 256, 0, st>>>(t, hd, dim, pr->dx[0], pr->dx[1], pr->dx[2], p->hzt64, p->hzcol);
             PD_LAUNCH_CHECK();
@@ -1058,21 +1076,15 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
             const double sn[8] = {0, r2, 1, r2, 0, -r2, -1, -r2};
             t64[k] = mk(cs[o], -sn[o]);
         }
-        // the tables of every length and stage radix (pd_cols.cuh)
+        // the tables of every length and stage radix (pd_cols.cuh), made on the device
+        // from the longest plain table
         const int ne = tw_entries(p->lgl);
-        std::vector<cx<double>> a64(ne, mk(1.0, 0.0));
-        std::vector<cx<float>> a32(ne);
-        for (int k = 0; k <= p->lgl; ++k)
-            for (int r = 0; r < kTwRadices; ++r)
-                for (int i = 0; i < (1 << k) && r <= k; ++i) {
-                    const int e = r ? (i >> r) * (i & ((1 << r) - 1)) : i;  // j q at j 2^r + q
-                    a64[tw_base(k, r) + i] = t64[e << (p->lgl - k)];
-                }
-        for (int i = 0; i < ne; ++i) a32[i] = mk((float)a64[i].x, (float)a64[i].y);
         PD_TRY(dalloc(p, &p->tw64, sizeof(cx<double>) * ne));
         PD_TRY(dalloc(p, &p->tw32, sizeof(cx<float>) * ne));
-        PD_CUDA_TRY(cudaMemcpyAsync(p->tw64, a64.data(), sizeof(cx<double>) * ne, cudaMemcpyHostToDevice, st));
-        PD_CUDA_TRY(cudaMemcpyAsync(p->tw32, a32.data(), sizeof(cx<float>) * ne, cudaMemcpyHostToDevice, st));
+        PD_CUDA_TRY(cudaMemcpyAsync(p->tw64 + tw_base(p->lgl, 0), t64.data(), sizeof(cx<double>) * L,
+                                    cudaMemcpyHostToDevice, st));
+        k_twiddles<<<nblk(ne, 256), 256, 0, st>>>(p->lgl, p->tw64, p->tw32);
+        PD_LAUNCH_CHECK();
         PD_CUDA_TRY(cudaStreamSynchronize(st));
     }
 

@@ -51,7 +51,6 @@ namespace {
 
 constexpr int kHostStatus = 32;  // slot of the pinned host scalars that receives the device status word
 
-// rr = sum of the first pass's partials; alpha, beta from the second pass's triples
 // rr = sum of the first pass's partials; alpha, beta from the second pass's
 // triples (one block of kFinishThreads)
 __global__ void __launch_bounds__(kFinishThreads) k_cg_finish_fused(double *red, int na, int nb)
@@ -59,8 +58,10 @@ __global__ void __launch_bounds__(kFinishThreads) k_cg_finish_fused(double *red,
     pdl_wait();
     pdl_trigger();
     double rr = 0.0, pq = 0.0, rq = 0.0, qq = 0.0;
-    for (int i = threadIdx.x; i < na; i += blockDim.x) rr += red[kRedPart + i];
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < na; i += kFinishThreads) rr += red[kRedPart + i];
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nb; i += kFinishThreads) {
         pq += red[kRedPart + kPartB + 3 * i];
         rq += red[kRedPart + kPartB + 3 * i + 1];
         qq += red[kRedPart + kPartB + 3 * i + 2];

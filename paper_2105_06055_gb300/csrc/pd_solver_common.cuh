@@ -14,17 +14,22 @@ constexpr int kUpdBlocks = 1024;  // blocks of the vector kernels
 enum { S_RR = 0, S_PQ, S_ALPHA, S_BETA, S_RRNEW, S_NORM, S_BN, S_FLAG, S_COUNT };
 
 // Sum of four doubles per thread over a block of kFinishThreads threads
-// (valid in thread 0): warp shuffles, one shared-memory exchange.
-constexpr int kFinishThreads = 256;
+// (valid in thread 0): warp shuffles, one shared-memory exchange, the sums of
+// the warps by the first warp's shuffles. (With 256 threads, loads one after the
+// other and thread 0 adding up the warps, the CG's finish kernel took 10.1 us in a
+// 128^3 iteration's launch list.)
+constexpr int kFinishThreads = 512;
 __device__ __forceinline__ void block_sum4(double &a, double &b, double &c, double &d)
 {
-    __shared__ double sh[4][kFinishThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-        d += __shfl_down_sync(0xffffffffu, d, o);
-    }
+    constexpr int W = kFinishThreads / 32;
+    __shared__ double sh[4][W];
+    auto warp_sum = [](double &x, int n) {
+        for (int o = n / 2; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    };
+    warp_sum(a, 32);
+    warp_sum(b, 32);
+    warp_sum(c, 32);
+    warp_sum(d, 32);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) {
         sh[0][wid] = a;
@@ -33,14 +38,15 @@ __device__ __forceinline__ void block_sum4(double &a, double &b, double &c, doub
         sh[3][wid] = d;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        a = b = c = d = 0.0;
-        for (int k = 0; k < kFinishThreads / 32; ++k) {
-            a += sh[0][k];
-            b += sh[1][k];
-            c += sh[2][k];
-            d += sh[3][k];
-        }
+    if (wid == 0) {
+        a = lane < W ? sh[0][lane] : 0.0;
+        b = lane < W ? sh[1][lane] : 0.0;
+        c = lane < W ? sh[2][lane] : 0.0;
+        d = lane < W ? sh[3][lane] : 0.0;
+        warp_sum(a, W);
+        warp_sum(b, W);
+        warp_sum(c, W);
+        warp_sum(d, W);
     }
 }
 
