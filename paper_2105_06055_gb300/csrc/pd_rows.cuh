@@ -34,10 +34,11 @@ namespace pd {
 
 // Chunk radix (log2) of a row of 2^lg packed values: 8, a lane then holds 16
 // values; 4 (8 values a lane, twice the lanes per row) for FP64 and for the 2D
-// grids up to 256 nodes wide. Both have few warps for the chip otherwise: a
-// 128 x 128 plate in FP64 has 256 row transforms, and a warp's FP64 instructions,
-// 64 clocks each, ran one after the other on 8 of the SMs (23 us a pass).
-__host__ __device__ constexpr int row_lgc(bool fp64, int dim, int lg) { return (fp64 || dim == 2) && lg <= 7 ? 2 : 3; }
+// grids up to 512 nodes wide. Both have few warps for the chip otherwise: a
+// 128 x 128 plate in FP64 has 256 row transforms, and a warp's FP64 instructions
+// ran one after the other on 8 of the SMs (force 71 us, now 53; 512 x 128: 102,
+// now 79; 512 x 1024 in FP32: 43, now 35).
+__host__ __device__ constexpr int row_lgc(bool fp64, int dim, int lg) { return (fp64 || dim == 2) && lg <= 8 ? 2 : 3; }
 
 // Row transform of 2^LG packed values: stages RA (RB) RC.
 template <int LG, int LGC_>
