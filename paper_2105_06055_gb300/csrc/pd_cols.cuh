@@ -230,7 +230,6 @@ __global__ void __launch_bounds__(PlainShape<T, LG, INV>::THREADS)
     // uniform base + 32-bit lane offset (a slot is below 2^32 values)
     cx<T> *p = g.spec + (slot0 + (int)blockIdx.z) * g.fs + blockIdx.y * g.os + (int64_t)blockIdx.x * S::W;
     const unsigned ls = (unsigned)g.ls;
-    pdl_trigger();
     pdl_wait();
     auto chunk_pass = [&]() {
 #pragma unroll
@@ -359,7 +358,6 @@ __global__ void __launch_bounds__(CombShape<T, Op, LG>::THREADS, comb_blocks<T, 
     }
     const unsigned ls = (unsigned)g.ls;
     const int64_t step = (int64_t)S::M * ls;
-    pdl_trigger();
     pdl_wait();
 
     // first stage: global -> registers -> shared. With few fields all of a

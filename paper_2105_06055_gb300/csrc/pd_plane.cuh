@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
     const int j = blockIdx.x % D, z = blockIdx.x / D;
     for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[tw_base(S::LGT, 0) + i];
     pdl_wait();
-    pdl_trigger();
 
     const int64_t base = (int64_t)z * S::n2 * S::n1 + (int64_t)j * a.N;
     const T alpha = (T)a.red[kRedScal + S_ALPHA], beta = (T)a.red[kRedScal + S_BETA];
@@ -221,7 +220,6 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
     for (int i = tid; i < (1 << S::LGT); i += S::THREADS) tws[i] = tw[tw_base(S::LGT, 0) + i];
     __syncthreads();
     pdl_wait();
-    pdl_trigger();
     if (tid == 0) {
         // test hook: one-shot, so a pass captured in a graph stalls on one replay only
         const bool stall = a.inject && blockIdx.x == 0 && atomicCAS(a.inject, 6, 0) == 6;

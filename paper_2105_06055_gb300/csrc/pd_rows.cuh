@@ -416,7 +416,6 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
     const int64_t ntiles = g.nrows / rows;
     constexpr bool kLoad = FI > 0 || NB > 0;
     if (kLoad && tid == 0) mbar_init(mbar, 1);
-    pdl_trigger();
     pdl_wait();
     if constexpr (kLoad) __syncthreads();  // the barrier is initialised
     bool stall = false;
