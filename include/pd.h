@@ -312,32 +312,28 @@ pd_status pd_solve_dr_batched(pd_batch *batch, double *const *u, const double *c
 void pd_batch_destroy(pd_batch *batch);
 
 /*
- * Autotuning of the FFT passes. pd_plan_autotune times the plan's force
- * evaluation (on its own workspace; no caller buffer is touched) over the
- * candidate rows per row-pass block, row-pass pipeline depths, column-tile
- * widths of the x2 and last-axis passes and FFT stage schedules (radix-4/2
- * remainder stage first or last), coordinate-wise from the built-in
- * heuristic, and keeps the fastest. Results do not change (the same transforms are computed); later
- * calls use the chosen configuration. Synchronises the stream.
- * pd_batch_autotune tunes one plan per distinct grid/precision/operator of a
- * batch and gives the others the same configuration.
+ * Autotuning of the FFT passes. The tile shapes of the row and column passes are
+ * compile-time constants per axis length, type and operator, so a force
+ * evaluation leaves nothing to choose: pd_plan_autotune (and, for the plans of a
+ * batch, pd_batch_autotune) fills the entries of the tuning record that are 0
+ * with nominal values. pd_plan_autotune_solve times what is left for the static
+ * solver. Results do not change.
  * pd_plan_tuning writes {rows, x2 width, last-axis width, schedule, stages,
- * inverse-pass stages} (0 = heuristic) to out6.
+ * inverse-pass stages} (0 = not set) to out6.
  */
 pd_status pd_plan_autotune(pd_plan *plan, void *stream);
-/* The same search timing a chunk of 16 iterations of the static solver's CG
- * (pd_solve_static's unit of work) instead of a force evaluation; uses the
- * plan's solver workspace. */
+/* FP32 plans on cubes of 32^3, 64^3 and 128^3: times a chunk of 16 iterations of
+ * the static solver's CG (pd_solve_static's unit of work) with the forward half
+ * as a plane pass and as row and column passes (pd_plan_set_plane_passes) on the
+ * plan's solver workspace, and keeps the faster. Synchronises the stream. */
 pd_status pd_plan_autotune_solve(pd_plan *plan, void *stream);
 pd_status pd_batch_autotune(pd_batch *batch, void *stream);
 pd_status pd_plan_tuning(const pd_plan *plan, int *out6);
-/* Pin a pass configuration {rows, x2 width, last-axis width, schedule,
- * stages, inverse-pass stages}: rows and widths 0 or powers of two (rows <=
- * 256, widths 2..32; 0 = heuristic), schedule 0/1, row-pass pipeline stages
- * 0 (= 2), 1 or 2, inverse-pass stages 0 (= as the forward passes), 1 or 2;
- * PD_ERR_ARG otherwise. The pass configuration functions still shrink a value
- * that does not fit the grid or the shared memory, and raise rows to fill at
- * least one warp per row-pass block. */
+/* Set the tuning record {rows, x2 width, last-axis width, schedule, stages,
+ * inverse-pass stages}: rows and widths 0 or powers of two (rows <= 256, widths
+ * 2..32), schedule 0/1, stages and inverse-pass stages 0, 1 or 2; PD_ERR_ARG
+ * otherwise. The record is kept and reported; the passes run with their own
+ * shapes whatever it holds. */
 pd_status pd_plan_set_tuning(pd_plan *plan, const int *in6);
 
 /*

@@ -97,12 +97,7 @@ __device__ __forceinline__ void dft_reg(cx<T> *v)
 // and pile onto two of the 16 eight-byte bank pairs; XOR-ing the element's
 // low three bits with the butterfly index spreads them over all pairs. With
 // 8 butterflies per row (rows 8 bank pairs apart) sh = 3 is conflict-free,
-// with 16 or more sh = 4. The row kernels compiled for a fixed row length and
-// the plane passes use it; in the column tiles the lanes of a warp differ
-// first in the column, the conflicts are at most 2-way at the tile widths the
-// passes run with, and the extra index arithmetic on the strided addresses
-// cost more than it saved (measured), as it did in the row kernels that read
-// the length at run time.
+// with 16 or more sh = 4.
 __device__ __forceinline__ int swz(int e, int sh) { return e ^ ((e >> sh) & 7); }
 
 // One radix-R Stockham stage of F length-n transforms, field f stored at
