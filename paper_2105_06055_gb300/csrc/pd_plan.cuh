@@ -353,7 +353,7 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     const auto kern = whole ? rows_kernel<T, Op>(g.lgh) : &k_rows<T, Op>;
     PD_TRY(set_smem_attr((const void *)kern, smem));
     PD_TRY(prof_begin(p, Op::kFin > 0 ? PASS_ROWS_INV : PASS_ROWS_FWD, st));
-    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(FB, lgc)), smem, st, g, op,
+    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(p->h, lgc, FB)), smem, st, g, op,
                     tw_buf<T>(p)));
     PD_TRY(prof_end(p, st));
     p->launches++;

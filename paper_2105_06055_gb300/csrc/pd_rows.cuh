@@ -40,49 +40,65 @@ namespace pd {
 // now 79; 512 x 1024 in FP32: 43, now 35).
 __host__ __device__ constexpr int row_lgc(bool fp64, int dim, int lg) { return (fp64 || dim == 2) && lg <= 8 ? 2 : 3; }
 
+// Lanes of a row: one row of 1024 packed values takes two warps (a named barrier
+// in place of the warp barrier), all others a warp or part of one. With 32 values
+// per lane the passes were a chain of one warp's instructions (force 2048 x 64 28 us,
+// now 20; 2048 x 512 43, now 36).
+__host__ __device__ constexpr int row_lanes(int H, int lgc)
+{
+    return (H >> (lgc + 1)) < 32 ? H >> (lgc + 1) : H >= 1024 ? 64 : 32;
+}
+// barrier of the lanes of a row (and of the other rows of their warp)
+template <int NT>
+__device__ __forceinline__ void row_sync()
+{
+    if constexpr (NT > 32)
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / NT), "n"(NT) : "memory");
+    else
+        __syncwarp();
+}
+
 // Row transform of 2^LG packed values: stages RA (RB) RC.
 template <int LG, int LGC_>
 struct RowShape {
     static constexpr int H = 1 << LG;
     static constexpr int LGC = LGC_, RC = 1 << LGC;
-    static constexpr int NT = H / (2 * RC) < 32 ? H / (2 * RC) : 32;  // lanes per row
+    static constexpr int NT = row_lanes(H, LGC);  // lanes per row
     static constexpr int V = H / NT;
-    static constexpr int REM = LG - LGC, LGV = LG - (NT == 32 ? 5 : LG - LGC - 1);
+    static constexpr int REM = LG - LGC, LGV = LG - (NT == 64 ? 6 : NT == 32 ? 5 : LG - LGC - 1);
     static constexpr int LGA = REM <= LGV && REM <= 4 ? REM : (REM + 1) / 2;
     static constexpr int LGB = REM - LGA;
     static constexpr int RA = 1 << LGA, RB = 1 << LGB, M = H / RA, K = H / RC;
     static constexpr int MP = M + M / RC;  // first-stage stride with the pad elements
-    static constexpr int ROWS = 32 / NT;   // rows of a warp
     static constexpr int PAIRS = K / 2 / NT;
     static_assert(LG >= 4 && LG <= 10 && PAIRS >= 1 && RA <= V && RB <= V && M % RC == 0, "row length");
 };
 // pitch of a padded row in shared memory (complex elements; even: rows start on
-// 16-byte boundaries), lanes per row and rows of a warp
-__host__ __device__ constexpr int row_lanes(int H, int lgc) { return (H >> (lgc + 1)) < 32 ? H >> (lgc + 1) : 32; }
+// 16-byte boundaries), rows of a warp or of a pair of warps
 __host__ __device__ constexpr int row_pitch(int H, int lgc)
 {
     const int nt = row_lanes(H, lgc);
     return H + (H >> lgc) + (nt >= 16 ? 0 : nt == 1 ? 2 : nt);
 }
-__host__ __device__ constexpr int row_warp_rows(int H, int lgc) { return 32 / row_lanes(H, lgc); }
+__host__ __device__ constexpr int row_warp_rows(int H, int lgc) { return row_lanes(H, lgc) < 32 ? 32 / row_lanes(H, lgc) : 1; }
 template <int LGC>
 __device__ __forceinline__ int row_at(int e)
 {
     return e + (e >> LGC);
 }
 // a tile holds the rows one warp transforms at a time, more of them for one
-// or two fields, and a warp per field and such group up to twelve
+// or two fields, and a warp (or pair) per field and such group, up to twelve warps
 __host__ __device__ constexpr int row_groups(int fields, int lgc) { return fields == 1 ? 4 : fields == 2 && lgc == 3 ? 2 : 1; }
 __host__ __device__ constexpr int row_tile_rows(int H, int lgc, int fields)
 {
     return row_warp_rows(H, lgc) * row_groups(fields, lgc);
 }
-__host__ __device__ constexpr int row_warps(int fields, int lgc)
+__host__ __device__ constexpr int row_warps(int H, int lgc, int fields)
 {
-    const int tasks = fields * row_groups(fields, lgc);
+    const int tasks = fields * row_groups(fields, lgc), pair = row_lanes(H, lgc) > 32 ? 2 : 1;
     int w = tasks;
-    for (int k = 2; w > 12; ++k) w = (tasks + k - 1) / k;
-    return w;
+    for (int k = 2; w * pair > 12; ++k) w = (tasks + k - 1) / k;
+    return w * pair;
 }
 
 // chunk index (shared-memory order) of mode residue m: m = q + RA q', chunk q RB + q'
@@ -130,10 +146,10 @@ __device__ __forceinline__ void row_forward(unsigned so, bool on, int t, const c
 #pragma unroll
         for (int r = 0; r < S::RA; ++r) s[o + r * S::MP] = v[r];
     }
-    __syncwarp();
+    row_sync<S::NT>();
     if constexpr (S::RB > 1) {
         if (on) row_stage_b<T, S, LG, false>(s, t, tw);
-        __syncwarp();
+        row_sync<S::NT>();
     }
     // all chunks into registers before the spectrum overwrites them
     cx<T> z[S::PAIRS][S::RC], y[S::PAIRS][S::RC];
@@ -147,7 +163,7 @@ __device__ __forceinline__ void row_forward(unsigned so, bool on, int t, const c
 #pragma unroll
         for (int k = 0; k < S::RC; ++k) y[b][k] = s[cb + k];
     }
-    __syncwarp();
+    row_sync<S::NT>();
 #pragma unroll
     for (int b = 0; on && b < S::PAIRS; ++b) {
         const int m = t + b * S::NT;
@@ -201,7 +217,7 @@ __device__ __forceinline__ void row_inverse(unsigned so, bool on, int t, const c
 #pragma unroll
         for (int k = 0; k < S::RC; ++k) c[b][k] = s[S::H - ((k < C2 ? lo : m) + S::K * k)];
     }
-    __syncwarp();  // the spectrum is in registers; the chunks overwrite it
+    row_sync<S::NT>();  // the spectrum is in registers; the chunks overwrite it
 #pragma unroll
     for (int b = 0; on && b < S::PAIRS; ++b) {
         const int m = t + b * S::NT, lo = m ? m : S::K / 2, mm = m ? S::K - m : S::K / 2;
@@ -237,10 +253,10 @@ __device__ __forceinline__ void row_inverse(unsigned so, bool on, int t, const c
 #pragma unroll
         for (int k = 0; k < S::RC; ++k) s[cb + k] = y[k];
     }
-    __syncwarp();
+    row_sync<S::NT>();
     if constexpr (S::RB > 1) {
         if (on) row_stage_b<T, S, LG, true>(s, t, tw);
-        __syncwarp();
+        row_sync<S::NT>();
     }
     if (!on) return;
 #pragma unroll
@@ -384,8 +400,8 @@ constexpr int kRowThreads = 384;
 template <typename T, class Op, int LG>
 constexpr int row_threads()
 {
-    return LG > 0 ? 32 * row_warps(Op::kFin > Op::kFout ? Op::kFin : Op::kFout, row_lgc(sizeof(T) == 8, Op::kDim, LG))
-                  : kRowThreads;
+    constexpr int FB = Op::kFin > Op::kFout ? Op::kFin : Op::kFout;
+    return LG > 0 ? 32 * row_warps(1 << LG, row_lgc(sizeof(T) == 8, Op::kDim, LG), FB) : kRowThreads;
 }
 template <typename T, class Op, int LG>
 constexpr int row_blocks()
@@ -406,13 +422,14 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
     uint8_t *nb = smem_raw + 16;
     const unsigned spec_off = 16u + (unsigned)(NB * rows * n1);
     cx<T> *spec = reinterpret_cast<cx<T> *>(smem_raw + spec_off);
-    const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
-    const int nt = row_lanes(H, lgc), wr = 32 / nt;  // lanes of a row, rows of a warp
+    const int tid = threadIdx.x;
+    const int nt = row_lanes(H, lgc), tl = nt < 32 ? 32 : nt, wr = tl / nt;  // lanes of a row, of a task; its rows
+    const int task0 = tid / tl, ntask = (int)blockDim.x / tl;
     auto at = [&](int e) { return e + (e >> lgc); };
     const int fstr = rows * pitch;  // field stride of the tile
     // node pairs loaded ahead: about 36 registers' worth
     constexpr int U0 = (int)(144 / sizeof(typename Op::Nd)), U = U0 < 1 ? 1 : U0 > 6 ? 6 : U0;
-    const int lr = lane / nt, lt = lane & (nt - 1), groups = LG > 0 ? row_groups(FB, lgc) : rows > wr ? rows / wr : 1;
+    const int lr = (tid & (tl - 1)) / nt, lt = tid & (nt - 1), groups = LG > 0 ? row_groups(FB, lgc) : rows > wr ? rows / wr : 1;
     const int64_t ntiles = g.nrows / rows;
     constexpr bool kLoad = FI > 0 || NB > 0;
     if (kLoad && tid == 0) mbar_init(mbar, 1);
@@ -462,7 +479,7 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
         if constexpr (FI > 0) {
             if (!arrive()) return;
 #pragma unroll 1
-            for (int task = tid >> 5; task < FI * groups; task += nw) {
+            for (int task = task0; task < FI * groups; task += ntask) {
                 const int f = task / groups, r = (task - f * groups) * wr + lr;
                 const unsigned s = spec_off + (unsigned)((f * rows + r) * pitch) * (unsigned)sizeof(cx<T>);
                 const bool on = r < rows;
@@ -486,7 +503,7 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
             }
         }
         const RowCtx ctx{row0, row0 * n1, rows * n1, nb};
-        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(FB, lgc) : (int)blockDim.x;
+        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(H, lgc, FB) : (int)blockDim.x;
         typename Op::Nd nd[U];
         auto load = [&](int i0) {
 #pragma unroll
@@ -522,13 +539,16 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
         if constexpr (FO > 0) {
             __syncthreads();
 #pragma unroll 1
-            for (int task = tid >> 5; task < FO * groups; task += nw) {
+            for (int task = task0; task < FO * groups; task += ntask) {
                 const int f = task / groups, r = (task - f * groups) * wr + lr;
                 const unsigned s = spec_off + (unsigned)((f * rows + r) * pitch) * (unsigned)sizeof(cx<T>);
                 const bool on = r < rows;
                 row_transform<T, Op::kDim, LG, false>(lgh, s, LG > 0 || on, lt, tw);
                 fence_proxy_async();
-                __syncwarp();
+                if (nt > 32)
+                    row_sync<64>();
+                else
+                    __syncwarp();
                 if (lt == 0 && on) {
                     bulk_store(op.spec_out(f) + (row0 + r) * H, spec + (f * rows + r) * pitch,
                                (unsigned)(H * sizeof(cx<T>)));
