@@ -49,16 +49,50 @@ struct AffineView {
     }
 };
 
+// Body sums of a warp's lanes. A lane's FP32 sum is a pair (hi, lo); the lanes
+// are merged as triples, every addition's rounding error kept in the next term
+// by the two-sum (only the errors of the third, about 2^-70 of the sum, are
+// dropped), and one lane makes the FP64 sum of them. The warp's sum is so the
+// FP64 rounding of the lanes' pairs, as if they had been converted and added in
+// FP64, without that pipe: it runs at 1/64 of the FP32 rate, and a block
+// reduction in FP64 per sum kept it busy for 60 us of a 64^3 evaluation. Merged
+// as pairs, the sums carried about 48 bits (64^3 nonlinear force 68.7 us, with
+// triples 70.4).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = a + b;
+    const float bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+}
+__device__ __forceinline__ double warp_body_sum(const DSum &a)
+{
+    float hi = a.hi, lo = a.lo, l3 = 0.f;
+    double d = a.d;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+        const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        l3 += __shfl_xor_sync(0xffffffffu, l3, o);
+        float e, f, g;
+        two_sum(hi, h2, hi, e);
+        two_sum(lo, l2, lo, f);
+        two_sum(lo, e, lo, g);
+        l3 += f + g;
+    }
+    if (__any_sync(0xffffffffu, d != 0.0))
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    return d + ((double)hi + ((double)lo + (double)l3));
+}
+
 // Block partial sums of the fit: Σ chi u_j (D values) and Σ chi e_k u_j
 // (D^2 values, index D + D j + k), in compensated FP32 (FP64 for FP64 fields).
-// NV = D: the first D sums only (the body mean). One block_sums exchange for
-// all sums: FP32 pairs are merged per warp and only one lane per warp and sum
-// touches FP64 (a separate FP64 block reduction per sum kept the FP64 pipe busy
-// for 60 us of a 64^3 evaluation).
+// NV = D: the first D sums only (the body mean). One exchange between the warps
+// for all sums.
 template <typename T, int D, int NV = D + D * D>
 __global__ void __launch_bounds__(256) k_aff_sums(const T *u, const uint8_t *chi, int lg1, int lg2, int c0, int c1,
                                                   int c2, int64_t N, double *red)
 {
+    __shared__ double part[8][NV];
     DSum acc[NV];
     pdl_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
@@ -76,14 +110,17 @@ __global__ void __launch_bounds__(256) k_aff_sums(const T *u, const uint8_t *chi
         }
     }
     pdl_trigger();
-    const DSum *a[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) a[v] = &acc[v];
-    double t[NV];
-    block_sums<NV>(a, t);
-    if (threadIdx.x == 0) {
+    for (int v = 0; v < NV; ++v) {
+        const double t = warp_body_sum(acc[v]);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][v] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double t = 0.0;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) red[kRedPart + (int64_t)blockIdx.x * NV + v] = t[v];
+        for (int k = 0; k < 8; ++k) t += part[k][threadIdx.x];
+        red[kRedPart + (int64_t)blockIdx.x * NV + threadIdx.x] = t;
     }
 }
 
