@@ -230,8 +230,10 @@ __global__ void __launch_bounds__(PlaneShape<T, LGH, LG2>::THREADS, 3)
                 bulk_load(pl + y * S::PITCH, src + (int64_t)y * S::H, S::H * sizeof(cx<T>), mbar);
         }
     }
-    const bool ok = mbar_wait(mbar, 0, a.err);
-    if (__syncthreads_or(!ok)) return;  // no copy in flight: the stalled block issued none
+    if (!wait_for_copies(
+            tid == 0, [&]() { return mbar_wait(mbar, 0, a.err); }, [](bool x) { return __syncthreads_or(x) != 0; },
+            [&]() { mbar_drain(smem_u32(mbar), 0); }))
+        return;
     if (tid == 0) {
         // p_j, r_j and the mask bytes towards L2 while the plane is transformed
         // (issued once the spectrum is in, so they do not compete with it)

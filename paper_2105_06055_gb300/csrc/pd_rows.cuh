@@ -470,11 +470,13 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
             k0 = op.rows_off()[row0];
             k1 = op.rows_off()[row0 + rows];
         }
-        // false: the wait ran out (no copy is in flight then: the stalled block issued none)
+        // false: the wait ran out
         auto arrive = [&]() {
-            const bool ok = mbar_wait(mbar, phase, g.err);
+            const bool ok = wait_for_copies(
+                tid == 0, [&]() { return mbar_wait(mbar, phase, g.err); },
+                [](bool x) { return __syncthreads_or(x) != 0; }, [&]() { mbar_drain(smem_u32(mbar), phase); });
             phase ^= 1u;
-            return !__syncthreads_or(!ok);
+            return ok;
         };
         if constexpr (FI > 0) {
             if (!arrive()) return;

@@ -3,7 +3,8 @@
 // Rows move between global and shared memory with cp.async.bulk (loads complete
 // on an mbarrier, stores drain through a bulk group). Every wait on an mbarrier
 // is bounded by the global timer: on time-out the block sets a bit in the plan's
-// device status word and leaves without touching the tile.
+// device status word, gives its copies as long again to land (they write to shared
+// memory that the SM hands to another block) and leaves without touching the tile.
 #pragma once
 
 #include "pd_common.cuh"
@@ -37,7 +38,7 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned long long *mbar, unsigne
                  : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *mbar, unsigned phase)
+__device__ __forceinline__ bool mbar_try_wait(unsigned mbar, unsigned phase)
 {
     unsigned ok;
     asm volatile(
@@ -45,7 +46,7 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *mbar, unsigned
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(mbar)), "r"(phase)
+        : "r"(mbar), "r"(phase)
         : "memory");
     return ok != 0;
 }
@@ -54,15 +55,40 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *mbar, unsigned
 // (after recording it in *err).
 __device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, unsigned phase, int *err)
 {
-    if (mbar_try_wait(mbar, phase)) return true;
+    const unsigned m = smem_u32(mbar);
+    if (mbar_try_wait(m, phase)) return true;
     const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(mbar, phase)) {
+    while (!mbar_try_wait(m, phase)) {
         if (global_ns() - t0 > kWaitLimitNs) {
             if (err) atomicOr(err, kErrTmaTimeout);
             return false;
         }
     }
     return true;
+}
+
+// The wait after one that ran out, bounded alike. Out of line: inlined it cost the row
+// passes up to 2% in registers and code (128^3 solve 0.6%, so 0.1%).
+static __device__ __noinline__ void mbar_drain(unsigned mbar, unsigned phase)
+{
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(mbar, phase) && global_ns() - t0 <= kWaitLimitNs) {
+    }
+}
+
+// A block's wait for the copies that its first thread has issued: wait() is one bounded
+// wait (false on time-out), vote(x) whether x holds in any thread of the block (a block
+// barrier). False when the wait of any thread ran out; the first thread has then
+// drained the copies, and the block leaves behind its second vote, together.
+template <class Wait, class Vote, class Drain>
+__host__ __device__ __forceinline__ bool wait_for_copies(bool first, Wait wait, Vote vote, Drain drain)
+{
+    const bool out = vote(!wait());
+    if (out) {
+        if (first) drain();
+        vote(false);
+    }
+    return !out;
 }
 
 // 1D bulk copy global -> shared (16-byte aligned addresses, size multiple of 16)
