@@ -8,11 +8,9 @@
 #include <cstring>
 #include <vector>
 
-#include <map>
-#include <mutex>
-
 #include "pd_horizon.cuh"
 #include "pd_plan.cuh"
+#include "pd_smem_limit.cuh"
 
 namespace pd {
 
@@ -26,24 +24,21 @@ void set_error(const char *fmt, ...)
     va_end(ap);
 }
 
-// The dynamic shared-memory limit is a property of the kernel function, shared
-// by every plan and by every kernel node of a captured graph: it only ever
-// grows, so plans of different sizes never lower it under each other.
+// Raises the dynamic shared-memory limit of a kernel on the current device (SmemLimits).
 pd_status set_smem_attr(const void *func, size_t smem)
 {
-    static std::mutex mu;
-    static std::map<const void *, size_t> set;
+    static SmemLimits limits;
     if (smem <= 48 * 1024) return PD_OK;
-    std::lock_guard<std::mutex> lock(mu);
-    size_t &cur = set[func];
-    if (smem <= cur) return PD_OK;
-    cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0;
+    PD_CUDA_TRY(cudaGetDevice(&dev));
+    const cudaError_t e = (cudaError_t)limits.raise(dev, func, smem, [&]() {
+        return (int)cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
     if (e != cudaSuccess) {
         set_error("cudaFuncSetAttribute(%zu bytes): %s", smem, cudaGetErrorString(e));
         cudaGetLastError();  // the call is refused; later launches are not
         return PD_ERR_CUDA;
     }
-    cur = smem;
     return PD_OK;
 }
 
