@@ -8,9 +8,9 @@ w = 0) on the three node layers at the x1-low face, body-force layer
 b1 = sigma/delta (sigma = 1e-3) on the three layers at the x1-high face.
 One step = one complete static solve from u = 0 to a relative FP64 residual of
 1e-8: FP32 FFT-convolution CG with FP64 inner products inside FP64 iterative
-refinement (pd_solve_static). The plan's pass configuration is picked by the
-library's autotuner timing the solver's own CG iterations
-(pd_plan_autotune_solve) before the warm-up, unless --no-autotune.
+refinement (pd_solve_static). The layout of the CG's passes (plane passes or row
+and column passes) is picked by the library's autotuner timing the solver's own
+CG iterations (pd_plan_autotune_solve) before the warm-up, unless --no-autotune.
 
 Metric: force evaluations x nodes per second (each CG iteration and each FP64
 residual is one evaluation of the PD operator on all 128^3 nodes), plus the
@@ -198,11 +198,7 @@ def run_native(args, rank, world):
     plan = pd.Plan(prob, chi, chi_om)
     if args.plane_mask is not None:
         plan.set_plane_passes(args.plane_mask)
-    if args.tuning:
-        plan.set_tuning(*[int(v) for v in args.tuning.split(",")])
-        tuning = plan.tuning
-    else:
-        tuning = None if args.no_autotune else plan.autotune(solve=True)
+    tuning = None if args.no_autotune else plan.autotune(solve=True)
     b = torch.tensor(cfg["b"], dtype=torch.float64, device=dev)
     u = torch.zeros((3,) + shape, dtype=torch.float64, device=dev)
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device=dev)  # 256 MB > L2
@@ -353,7 +349,7 @@ FORCE_PASS_BYTES = {  # algorithmic bytes per node of each FP32 pass of the bond
 }
 
 
-def force_point(n, steps, warmup, tuning_arg="", no_autotune=False, e2e=True):
+def force_point(n, steps, warmup, e2e=True):
     """One FP32 bond-model force evaluation (pd_force) on an n^3 box: median
     event time over `steps` evaluations (L2 flushed between them), per-pass
     event times and their algorithmic-byte fractions of the measured peak."""
@@ -367,11 +363,7 @@ def force_point(n, steps, warmup, tuning_arg="", no_autotune=False, e2e=True):
     chi = inputs.cube_with_ball_mask(n)
     u = inputs.separable_modes(shape, 4, max(n // 16, 2), 1e-3, seed=n, kmin=max(n // 32, 1)) * chi
     plan = pd.Plan(pd.Problem(shape=shape, delta=DELTA, fp64=False), torch.tensor(chi, device=dev))
-    if tuning_arg:
-        plan.set_tuning(*[int(v) for v in tuning_arg.split(",")])
-        tuning = plan.tuning
-    else:
-        tuning = None if no_autotune else plan.autotune()
+    tuning = plan.autotune()  # the passes' tile shapes
     ud = torch.tensor(u, device=dev)
     L = torch.empty_like(ud)
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device=dev)
@@ -446,7 +438,7 @@ def run_force(args):
     pd_build.build()
     n = args.n
     N = n ** 3
-    pt = force_point(n, args.steps, args.warmup, args.tuning, args.no_autotune)
+    pt = force_point(n, args.steps, args.warmup)
     passes = pt["passes"]
     dom = max(passes, key=lambda k: passes[k]["us"] * (2 if k == "cols_x2" else 1))
     traffic = MEASURED_TRAFFIC.get(f"force{n}_{dom}", (None, None))
@@ -640,12 +632,10 @@ def main():
     ap.add_argument("--n", "--grid", dest="n", type=int, default=N_GRID)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--workload", default="static", choices=["static", "batched", "force"])
-    ap.add_argument("--no-autotune", action="store_true", help="skip the pass autotuner (built-in tile heuristic)")
+    ap.add_argument("--no-autotune", action="store_true", help="static solve: skip the autotuner of the CG's pass layout (the library's default layout)")
     ap.add_argument("--plane-mask", type=int, default=None, metavar="M",
                     help="static solve: halves of the CG iteration run as fused x1-x2 plane passes (bit 0 forward, "
                          "bit 1 inverse; 0 = row and column passes; default: the library's)")
-    ap.add_argument("--tuning", default="", metavar="ROWS,WX2,WLAST,SCHED[,STAGES[,STAGES_INV]]",
-                    help="pin a pass configuration instead of autotuning (e.g. the one a tuned run reported)")
     ap.add_argument("--specimens", type=int, default=64)
     ap.add_argument("--no-sweep", dest="sweep", action="store_false",
                     help="skip the 256^3 / 512^3 force-evaluation keys of the default run")
@@ -666,9 +656,7 @@ def main():
                        torch.tensor(cfg["chi"], device=dev), torch.tensor(cfg["chi_omega"], device=dev))
         if args.plane_mask is not None:
             plan.set_plane_passes(args.plane_mask)
-        if args.tuning:
-            plan.set_tuning(*[int(v) for v in args.tuning.split(",")])
-        elif not args.no_autotune:
+        if not args.no_autotune:
             plan.autotune(solve=True)
         u = torch.zeros((3,) + cfg["shape"], dtype=torch.float64, device=dev)
         it, rel, _ = plan.solve_static(u, torch.tensor(cfg["b"], dtype=torch.float64, device=dev), None,
@@ -738,7 +726,7 @@ def main():
         # the headline stays the static solve)
         sweep = {}
         for n in (256, 512):
-            pt = force_point(n, 5, 3, "", args.no_autotune, e2e=False)
+            pt = force_point(n, 5, 3, e2e=False)
             sweep[f"{n}^3"] = {k: pt[k] for k in ("ms_per_eval", "node_evals_per_s", "passes",
                                                   "m2_end_to_end_hbm_frac", "tuning")}
         result["force_sweep"] = sweep

@@ -315,11 +315,13 @@ void pd_batch_destroy(pd_batch *batch);
  * Autotuning of the FFT passes. The tile shapes of the row and column passes are
  * compile-time constants per axis length, type and operator, so a force
  * evaluation leaves nothing to choose: pd_plan_autotune (and, for the plans of a
- * batch, pd_batch_autotune) fills the entries of the tuning record that are 0
- * with nominal values. pd_plan_autotune_solve times what is left for the static
- * solver. Results do not change.
- * pd_plan_tuning writes {rows, x2 width, last-axis width, schedule, stages,
- * inverse-pass stages} (0 = not set) to out6.
+ * batch, pd_batch_autotune) records the shapes that the passes of the plan's force
+ * evaluation run with. pd_plan_autotune_solve also times what is left for the
+ * static solver. Results do not change.
+ * pd_plan_tuning writes the record {rows per row tile, columns per x2 tile (0 in
+ * 2D, which has no such pass), columns per last-axis tile, schedule, stages,
+ * inverse-pass stages} to out6: all 0 on a new plan, then what an autotuner found or
+ * pd_plan_set_tuning stored, whichever came last.
  */
 pd_status pd_plan_autotune(pd_plan *plan, void *stream);
 /* FP32 plans on cubes of 32^3, 64^3 and 128^3: times a chunk of 16 iterations of
@@ -329,11 +331,10 @@ pd_status pd_plan_autotune(pd_plan *plan, void *stream);
 pd_status pd_plan_autotune_solve(pd_plan *plan, void *stream);
 pd_status pd_batch_autotune(pd_batch *batch, void *stream);
 pd_status pd_plan_tuning(const pd_plan *plan, int *out6);
-/* Set the tuning record {rows, x2 width, last-axis width, schedule, stages,
- * inverse-pass stages}: rows and widths 0 or powers of two (rows <= 256, widths
- * 2..32), schedule 0/1, stages and inverse-pass stages 0, 1 or 2; PD_ERR_ARG
- * otherwise. The record is kept and reported; the passes run with their own
- * shapes whatever it holds. */
+/* Store a record {rows, x2 width, last-axis width, schedule, stages, inverse-pass
+ * stages}: rows and widths 0 or powers of two (rows <= 256, widths 2..32), schedule
+ * 0/1, stages and inverse-pass stages 0, 1 or 2; PD_ERR_ARG otherwise. The passes
+ * run with their own shapes whatever it holds. */
 pd_status pd_plan_set_tuning(pd_plan *plan, const int *in6);
 
 /*

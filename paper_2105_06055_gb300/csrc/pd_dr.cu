@@ -878,14 +878,3 @@ extern "C" void pd_batch_destroy(pd_batch *B)
     B->plans.clear();
     delete B;
 }
-
-// forget the cached graph (the plans' pass configuration changed)
-void pd_batch_invalidate(pd_batch *B)
-{
-    if (B && B->runner.exec) {
-        cudaStreamSynchronize(B->runner.ms);
-        cudaGraphExecDestroy(B->runner.exec);
-        B->runner.exec = nullptr;
-        B->runner.key.clear();
-    }
-}

@@ -42,6 +42,7 @@ struct NL {
     static constexpr int INV = D + D * D + NS + D;   // P (D), A (D^2), B (NS), Cc (D)
     static constexpr int X = 0, Y = D, Z = D + NS;
     static constexpr int P = 0, A = D, B = D + D * D, CC = D + D * D + NS;
+    static_assert(FWD == kNLFwd<D> && INV == kNLInv<D>, "field counts");
 };
 
 // the body mean of u (from the block sums) as the coefficient t of

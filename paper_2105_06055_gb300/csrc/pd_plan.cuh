@@ -24,6 +24,13 @@ struct GEntry {
     int64_t p;
 };
 
+// Fields of a force evaluation of the nonlinear bond model: forward, inverse
+// (the linearized models: one per component)
+template <int D>
+constexpr int kNLFwd = 2 * D + D * (D + 1) / 2;
+template <int D>
+constexpr int kNLInv = D + D * D + D * (D + 1) / 2 + D;
+
 // Device-side view of the model used by the per-node and per-mode functors.
 template <typename T>
 struct Model {
@@ -194,7 +201,8 @@ struct pd_plan {
     // the larger ones (64^3: 38.3 against 41.4, 128^3: 108 against 122).
     int plane_passes = 0;
     double prof_ms[kKinds] = {};
-    // tuning record (pd_plan_tuning; the passes' shapes are constants per length)
+    // tuning record (pd_plan_tuning): pd_plan_set_tuning's, or the passes' shapes as an
+    // autotuner recorded them; the passes do not read it
     int tune_rows = 0;
     int tune_w[2] = {0, 0};
     int tune_sched = 0;
@@ -321,8 +329,18 @@ auto rows_kernel(int lgh)
     return (K)&k_rows<T, Op>;
 }
 
-// Row pass: tile and warps by row_tile_rows and row_warps (fewer rows when the
-// grid has fewer). Passes with block reductions run on at most 8 blocks per SM
+// Rows per tile of a row pass over `fields` fields: row_tile_rows, fewer when the grid
+// has fewer (*whole: the tile size the fixed-length kernels are compiled for).
+template <typename T, int D>
+int row_tile(const pd_plan *p, int fields, bool *whole)
+{
+    int rows = row_tile_rows(p->h, row_lgc(sizeof(T) == 8, D, ilog2(p->h)), fields);
+    *whole = p->nrows % rows == 0;
+    while (p->nrows % rows) rows >>= 1;
+    return rows;
+}
+
+// Row pass: tile by row_tile, warps by row_warps. Passes with block reductions run on at most 8 blocks per SM
 // (each block writes partial sums), all with as many tiles as far as it goes; the
 // others on a block per tile. *grid_out
 // receives the block count.
@@ -333,12 +351,8 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     RowGeom g;
     g.lgh = ilog2(p->h);
     const int lgc = row_lgc(sizeof(T) == 8, Op::kDim, g.lgh);
-    g.rows = row_tile_rows(p->h, lgc, FB);
-    bool whole = true;  // the tile size the fixed-length kernels are compiled for
-    while (p->nrows % g.rows) {
-        g.rows >>= 1;
-        whole = false;
-    }
+    bool whole = true;
+    g.rows = row_tile<T, Op::kDim>(p, FB, &whole);
     g.nrows = p->nrows;
     g.err = p->dev_status;
     g.inject = p->inject;

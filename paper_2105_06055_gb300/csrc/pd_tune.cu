@@ -6,17 +6,14 @@
 // The tile shapes of the row and column passes are compile-time constants per
 // axis length (pd_rows.cuh, pd_cols.cuh): with the length and the shape known
 // the index arithmetic folds away, which gained more than any choice of shape
-// at run time did. The tuning record (pd_plan_tuning, pd_plan_set_tuning) keeps
-// its six entries; autotuning reports the nominal shape in those that are 0.
-#include <map>
-#include <tuple>
-
+// at run time did. The tuning record (pd_plan_tuning) keeps its six entries: what
+// pd_plan_set_tuning stored, or, from an autotuner on, the shapes the passes of the
+// plan's force evaluation run with.
 #include "pd_plan.cuh"
 
 using namespace pd;
 
 struct pd_batch;
-void pd_batch_invalidate(pd_batch *B);
 extern "C" pd_plan *pd_batch_plan(pd_batch *B, int i);
 extern "C" int pd_batch_size(const pd_batch *B);
 
@@ -33,6 +30,59 @@ void drop_graphs(pd_plan *p)
             cudaGraphExecDestroy(p->cg_graph[k]);
             p->cg_graph[k] = nullptr;
         }
+}
+
+// Tile widths (columns) of the x2 pass and of the last-axis pass over FB fields.
+template <typename T>
+int x2_width(int lg)
+{
+    switch (lg) {
+        case 4: return PlainShape<T, 4, false>::W;
+        case 5: return PlainShape<T, 5, false>::W;
+        case 6: return PlainShape<T, 6, false>::W;
+        case 7: return PlainShape<T, 7, false>::W;
+        case 8: return PlainShape<T, 8, false>::W;
+        case 9: return PlainShape<T, 9, false>::W;
+        default: return PlainShape<T, 10, false>::W;
+    }
+}
+template <int D, int FB>
+struct Fields {
+    static constexpr int kFin = FB, kFout = FB, kDim = D;
+};
+template <typename T, class F>
+int last_width(int lg)
+{
+    switch (lg) {
+        case 4: return CombShape<T, F, 4>::W;
+        case 5: return CombShape<T, F, 5>::W;
+        case 6: return CombShape<T, F, 6>::W;
+        case 7: return CombShape<T, F, 7>::W;
+        case 8: return CombShape<T, F, 8>::W;
+        case 9: return CombShape<T, F, 9>::W;
+        default: return CombShape<T, F, 10>::W;
+    }
+}
+
+// The tuning record of the plan's force evaluation (without W): rows per tile of the
+// forward row pass, tile widths, one schedule, one tile at a time in the row passes.
+template <typename T, int D>
+void record_shapes(pd_plan *p)
+{
+    bool whole = true;
+    p->tune_rows = row_tile<T, D>(p, p->nonlinear ? kNLFwd<D> : D, &whole);
+    p->tune_w[0] = D == 3 ? x2_width<T>(ilog2(p->n2)) : 0;
+    const int lg = ilog2(D == 3 ? p->n3 : p->n2);
+    p->tune_w[1] = p->nonlinear ? last_width<T, Fields<D, kNLInv<D>>>(lg) : last_width<T, Fields<D, D>>(lg);
+    p->tune_sched = 0;
+    p->tune_stages = p->tune_stages_inv = 1;
+}
+void record_shapes(pd_plan *p)
+{
+    if (p->prob.fp64)
+        p->dim == 2 ? record_shapes<double, 2>(p) : record_shapes<double, 3>(p);
+    else
+        p->dim == 2 ? record_shapes<float, 2>(p) : record_shapes<float, 3>(p);
 }
 
 // target 1: the static solver's CG iteration, 0: force evaluations (nothing to choose)
@@ -72,11 +122,7 @@ pd_status tune_plan(pd_plan *p, cudaStream_t caller, int target = 0)
         PD_CUDA_TRY(cudaEventRecord(p->ev_join[1], p->own_stream));
         PD_CUDA_TRY(cudaStreamWaitEvent(caller, p->ev_join[1], 0));
     }
-    if (!p->tune_rows) p->tune_rows = row_warp_rows(p->h, row_lgc(p->prob.fp64 != 0, p->dim, ilog2(p->h)));
-    for (int k = 0; k < 2; ++k)
-        if (!p->tune_w[k]) p->tune_w[k] = p->prob.fp64 ? 8 : 16;
-    if (!p->tune_stages) p->tune_stages = 1;
-    if (!p->tune_stages_inv) p->tune_stages_inv = 1;
+    record_shapes(p);
     return PD_OK;
 }
 
@@ -126,26 +172,7 @@ extern "C" pd_status pd_batch_autotune(pd_batch *B, void *stream)
         set_error("pd_batch_autotune: null batch");
         return PD_ERR_ARG;
     }
-    // one search per distinct grid / precision / operator; the others copy it
-    std::map<std::tuple<int, int, int, int, int, int>, pd_plan *> done;
-    for (int i = 0; i < pd_batch_size(B); ++i) {
-        pd_plan *p = pd_batch_plan(B, i);
-        const auto key = std::make_tuple(p->dim, p->n1, p->n2, p->n3, p->prob.fp64, p->state_based);
-        auto it = done.find(key);
-        if (it == done.end()) {
-            PD_TRY(tune_plan(p, (cudaStream_t)stream));
-            done[key] = p;
-        } else {
-            p->tune_rows = it->second->tune_rows;
-            p->tune_w[0] = it->second->tune_w[0];
-            p->tune_w[1] = it->second->tune_w[1];
-            p->tune_sched = it->second->tune_sched;
-            p->tune_stages = it->second->tune_stages;
-            p->tune_stages_inv = it->second->tune_stages_inv;
-            drop_graphs(p);
-        }
-    }
-    pd_batch_invalidate(B);
+    for (int i = 0; i < pd_batch_size(B); ++i) PD_TRY(tune_plan(pd_batch_plan(B, i), (cudaStream_t)stream));
     return PD_OK;
 }
 
@@ -168,8 +195,7 @@ extern "C" pd_status pd_plan_set_tuning(pd_plan *p, const int *in6)
     }
     const int r = in6[0], wx = in6[1], wl = in6[2], sc = in6[3], ns = in6[4], ni = in6[5];
     auto pow2_or_zero = [](int v) { return v == 0 || (v > 0 && (v & (v - 1)) == 0); };
-    // a column tile is at least 2 complex values wide: its first column, and so the
-    // x coordinate of every tensor copy, is then a multiple of 16 bytes
+    // (a column tile is at least a pair of columns wide)
     if (!pow2_or_zero(r) || r > 256 || !pow2_or_zero(wx) || wx == 1 || wx > 32 || !pow2_or_zero(wl) || wl == 1 ||
         wl > 32 || (sc != 0 && sc != 1) || ns < 0 || ns > 2 || ni < 0 || ni > 2) {
         set_error("pd_plan_set_tuning: rows and widths must be 0 or powers of two (rows <= 256, widths 2..32), "
@@ -182,6 +208,5 @@ extern "C" pd_status pd_plan_set_tuning(pd_plan *p, const int *in6)
     p->tune_sched = sc;
     p->tune_stages = ns;
     p->tune_stages_inv = ni;
-    drop_graphs(p);
     return PD_OK;
 }

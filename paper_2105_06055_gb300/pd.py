@@ -383,8 +383,8 @@ class Plan:
         return int(it.value), float(rr.value), st
 
     def autotune(self, stream=None, solve=False):
-        """Fill the tuning record; with solve=True also pick the CG's pass layout by timing
-        chunks of the static solver's iterations."""
+        """Record the tile shapes that the plan's passes run with; with solve=True also pick
+        the CG's pass layout by timing chunks of the static solver's iterations."""
         if solve:
             _check(load().pd_plan_autotune_solve(self._h, _stream(stream)), "pd_plan_autotune_solve")
         else:
@@ -396,13 +396,13 @@ class Plan:
         _check(load().pd_plan_set_energy_mode(self._h, 1 if direct else 0), "pd_plan_set_energy_mode")
 
     def set_tuning(self, rows=0, w_x2=0, w_last=0, sched=0, stages=0, stages_inv=0):
-        """Set the tuning record (pd_plan_set_tuning)."""
+        """Store a tuning record (pd_plan_set_tuning); the passes do not read it."""
         arr = (ctypes.c_int * 6)(int(rows), int(w_x2), int(w_last), int(sched), int(stages), int(stages_inv))
         _check(load().pd_plan_set_tuning(self._h, arr), "pd_plan_set_tuning")
 
     @property
     def tuning(self):
-        """The tuning record {rows, w_x2, w_last, sched, stages, stages_inv} (0 = not set)."""
+        """The tuning record {rows, w_x2, w_last, sched, stages, stages_inv} (0 = not recorded)."""
         out = (ctypes.c_int * 6)()
         _check(load().pd_plan_tuning(self._h, out), "pd_plan_tuning")
         return {"rows": out[0], "w_x2": out[1], "w_last": out[2], "sched": out[3], "stages": out[4],
