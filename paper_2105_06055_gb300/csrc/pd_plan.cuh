@@ -334,7 +334,7 @@ auto rows_kernel(int lgh)
 template <typename T, int D>
 int row_tile(const pd_plan *p, int fields, bool *whole)
 {
-    int rows = row_tile_rows(p->h, row_lgc(sizeof(T) == 8, D, ilog2(p->h)), fields);
+    int rows = row_tile_rows(sizeof(T) == 8, p->h, row_lgc(sizeof(T) == 8, D, ilog2(p->h)), fields);
     *whole = p->nrows % rows == 0;
     while (p->nrows % rows) rows >>= 1;
     return rows;
@@ -367,8 +367,8 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
     const auto kern = whole ? rows_kernel<T, Op>(g.lgh) : &k_rows<T, Op>;
     PD_TRY(set_smem_attr((const void *)kern, smem));
     PD_TRY(prof_begin(p, Op::kFin > 0 ? PASS_ROWS_INV : PASS_ROWS_FWD, st));
-    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(p->h, lgc, FB)), smem, st, g, op,
-                    tw_buf<T>(p)));
+    PD_TRY(launch_k(p->pdl != 0, kern, dim3((unsigned)grid), dim3(32 * row_warps(sizeof(T) == 8, p->h, lgc, FB)), smem,
+                    st, g, op, tw_buf<T>(p)));
     PD_TRY(prof_end(p, st));
     p->launches++;
     return PD_OK;

@@ -87,15 +87,23 @@ __device__ __forceinline__ int row_at(int e)
     return e + (e >> LGC);
 }
 // a tile holds the rows one warp transforms at a time, more of them for one
-// or two fields, and a warp (or pair) per field and such group, up to twelve warps
-__host__ __device__ constexpr int row_groups(int fields, int lgc) { return fields == 1 ? 4 : fields == 2 && lgc == 3 ? 2 : 1; }
-__host__ __device__ constexpr int row_tile_rows(int H, int lgc, int fields)
+// or two fields, and a warp (or pair) per field and such group, up to twelve warps.
+// Two fields in FP64 and rows of 1024 packed values take one group: a block's warps
+// share one FP64 pipe and a grid of few rows has few blocks (2048 x 16: FP64 132 us
+// with two groups, 85 with one, 99 before the passes were rewritten; FP32 22.0, 18.3,
+// 17.9; larger grids at least as fast). FP32 rows of up to 512 keep two (1024 x 512
+// fracture steps: 1234 us, with one 1271).
+__host__ __device__ constexpr int row_groups(bool fp64, int H, int lgc, int fields)
 {
-    return row_warp_rows(H, lgc) * row_groups(fields, lgc);
+    return fields == 1 ? 4 : fields == 2 && lgc == 3 && !fp64 && H < 1024 ? 2 : 1;
 }
-__host__ __device__ constexpr int row_warps(int H, int lgc, int fields)
+__host__ __device__ constexpr int row_tile_rows(bool fp64, int H, int lgc, int fields)
 {
-    const int tasks = fields * row_groups(fields, lgc), pair = row_lanes(H, lgc) > 32 ? 2 : 1;
+    return row_warp_rows(H, lgc) * row_groups(fp64, H, lgc, fields);
+}
+__host__ __device__ constexpr int row_warps(bool fp64, int H, int lgc, int fields)
+{
+    const int tasks = fields * row_groups(fp64, H, lgc, fields), pair = row_lanes(H, lgc) > 32 ? 2 : 1;
     int w = tasks;
     for (int k = 2; w * pair > 12; ++k) w = (tasks + k - 1) / k;
     return w * pair;
@@ -401,7 +409,7 @@ template <typename T, class Op, int LG>
 constexpr int row_threads()
 {
     constexpr int FB = Op::kFin > Op::kFout ? Op::kFin : Op::kFout;
-    return LG > 0 ? 32 * row_warps(1 << LG, row_lgc(sizeof(T) == 8, Op::kDim, LG), FB) : kRowThreads;
+    return LG > 0 ? 32 * row_warps(sizeof(T) == 8, 1 << LG, row_lgc(sizeof(T) == 8, Op::kDim, LG), FB) : kRowThreads;
 }
 template <typename T, class Op, int LG>
 constexpr int row_blocks()
@@ -417,7 +425,7 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
     const int lgh = LG > 0 ? LG : g.lgh;
     const int lgc = row_lgc(sizeof(T) == 8, Op::kDim, lgh);
     const int H = 1 << lgh, n1 = 2 * H, pitch = row_pitch(H, lgc);
-    const int rows = LG > 0 ? row_tile_rows(H, lgc, FB) : g.rows;
+    const int rows = LG > 0 ? row_tile_rows(sizeof(T) == 8, H, lgc, FB) : g.rows;
     unsigned long long *mbar = reinterpret_cast<unsigned long long *>(smem_raw);
     uint8_t *nb = smem_raw + 16;
     const unsigned spec_off = 16u + (unsigned)(NB * rows * n1);
@@ -429,7 +437,8 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
     const int fstr = rows * pitch;  // field stride of the tile
     // node pairs loaded ahead: about 36 registers' worth
     constexpr int U0 = (int)(144 / sizeof(typename Op::Nd)), U = U0 < 1 ? 1 : U0 > 6 ? 6 : U0;
-    const int lr = (tid & (tl - 1)) / nt, lt = tid & (nt - 1), groups = LG > 0 ? row_groups(FB, lgc) : rows > wr ? rows / wr : 1;
+    const int lr = (tid & (tl - 1)) / nt, lt = tid & (nt - 1);
+    const int groups = LG > 0 ? row_groups(sizeof(T) == 8, H, lgc, FB) : rows > wr ? rows / wr : 1;
     const int64_t ntiles = g.nrows / rows;
     constexpr bool kLoad = FI > 0 || NB > 0;
     if (kLoad && tid == 0) mbar_init(mbar, 1);
@@ -505,7 +514,7 @@ __global__ void __launch_bounds__(row_threads<T, Op, LG>(), row_blocks<T, Op, LG
             }
         }
         const RowCtx ctx{row0, row0 * n1, rows * n1, nb};
-        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(H, lgc, FB) : (int)blockDim.x;
+        const int pairs = rows * H, nthr = LG > 0 ? 32 * row_warps(sizeof(T) == 8, H, lgc, FB) : (int)blockDim.x;
         typename Op::Nd nd[U];
         auto load = [&](int i0) {
 #pragma unroll
