@@ -126,6 +126,7 @@ struct ColArgs {
     int lgh;      // log2(n1/2)
     int n2;       // 3D last axis: n2; 2D last axis: 1 (one kx = 0 column, its own mirror)
     int nspec;    // special tiles (first blocks; 0 for the plain passes)
+    int sw;       // columns of a special tile on long axes (special_cols)
     int zaxis;    // 1: the transformed axis is x3
 };
 
@@ -312,11 +313,20 @@ constexpr int comb_blocks()
     return n < 1 ? 1 : n;
 }
 
-// Columns of a special tile: their elements are scattered 8- or 16-byte words
+// Columns of a special tile (pairs): their elements are scattered 8- or 16-byte words
 // (one L1 lookup each), so they are spread over more blocks than whole tiles
 // would make; with 16 columns these few blocks ran three times as long as the
-// others and set the pass's time at 128^3.
-constexpr int kSpecCols = 4;
+// others and set the pass's time at 128^3. On long axes of boxes whose other tiles fit
+// the SMs at once they still did with four (force on 32 x 16 x 1024 nodes in FP32: 84
+// us, with one pair a block 65, before the passes were rewritten 63; 32 x 16 x 512: 41.5
+// and 33.5): those take one pair. With more tiles the special ones end under the
+// others, and twice as many cost time (64 x 128 x 1024: 353 us, with one pair 368).
+// Below 512 nodes the two forms differ by a few us.
+constexpr int kSpecCols = 4, kLgLong = 9;
+__host__ __device__ constexpr int special_cols(int lg, int width, int64_t tiles, int nsm)
+{
+    return lg >= kLgLong && tiles <= nsm ? 2 : width < kSpecCols ? width : kSpecCols;
+}
 
 // Op of a combining pass:
 //   static constexpr int kFin, kFout, kTab;
@@ -343,7 +353,7 @@ __global__ void __launch_bounds__(CombShape<T, Op, LG>::THREADS, comb_blocks<T, 
     int kx, ky;
     bool active;
     if (special) {
-        constexpr int sw = S::W < kSpecCols ? S::W : kSpecCols;
+        const int sw = Op::kDim == 3 && LG >= kLgLong ? g.sw : special_cols(0, S::W, 0, 0);
         const int cc = (int)blockIdx.x * sw + c, k2 = cc >> 1;
         active = c < sw && k2 <= (g.n2 >> 1);
         ky = active ? k2 : 0;

@@ -389,6 +389,7 @@ inline ColArgs<T> col_args(const pd_plan *p, int zaxis)
     g.lgh = ilog2(p->h);
     g.n2 = zaxis ? p->n2 : 1;
     g.nspec = 0;
+    g.sw = 0;
     g.zaxis = zaxis;
     return g;
 }
@@ -415,10 +416,10 @@ pd_status launch_comb_lg(pd_plan *p, const Op &op, cudaStream_t st)
     PD_TRY(set_smem_attr((const void *)kern, S::smem));
     const int z = p->dim == 3 ? 1 : 0;
     ColArgs<T> g = col_args<T>(p, z);
-    // pairs of kx = 0 columns: k2 = 0 ... n2/2 in 3D, one column in 2D
-    constexpr int sw = S::W < kSpecCols ? S::W : kSpecCols;
-    g.nspec = ((z ? p->n2 + 2 : 2) + sw - 1) / sw;
     const unsigned tiles = (unsigned)((int64_t)(z ? p->n2 : 1) * p->h / S::W);
+    // pairs of kx = 0 columns: k2 = 0 ... n2/2 in 3D, one column in 2D
+    g.sw = z ? special_cols(LG, S::W, tiles, p->nsm) : special_cols(0, S::W, 0, 0);
+    g.nspec = ((z ? p->n2 + 2 : 2) + g.sw - 1) / g.sw;
     return launch_k(p->pdl != 0, kern, dim3(tiles + (unsigned)g.nspec), dim3(S::THREADS), S::smem, st, g, op,
                     tw_buf<T>(p));
 }
