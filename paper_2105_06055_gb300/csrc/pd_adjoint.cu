@@ -190,6 +190,7 @@ pd_status adjoint_pipeline(pd_plan *p, const T *u, const T *s, const T *pv, cons
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     constexpr int FI = 2 * D + Sym<D>::n, FO = 2 * D + 1;
+    PD_TRY(check_slots<T>(p, FI));
     const uintptr_t any = (uintptr_t)u | (uintptr_t)pv | (uintptr_t)s | (uintptr_t)gu | (uintptr_t)gs;
     const bool pairs = any % (2 * sizeof(T)) == 0;
     ProAdj<T, D> pro{u, pv, s, pairs, p->chi, p->N, p->n1, spec, fs};

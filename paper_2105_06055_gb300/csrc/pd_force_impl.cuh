@@ -46,6 +46,7 @@ pd_status force_bond_pipeline(pd_plan *p, const T *u, const T *s, const uint8_t 
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     constexpr int FI = D + (ENERGY ? Sym<D>::n : 0), FO = D + (ENERGY ? 1 : 0);
+    PD_TRY(check_slots<T>(p, FI));
     AffineView<T> av{};
     if (aff) PD_TRY((affine_fit<T, D>(p, u, st, &av)));
     const NodeWeight<T> w{s, lam};
@@ -209,6 +210,7 @@ pd_status force_state_pipeline(pd_plan *p, const T *u, T *L, T *theta, cudaStrea
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
     const Model<T> m = model_view<T>(p);
+    PD_TRY(check_slots<T>(p, 5));
     ProForce<T, 3, false> pro{u, NodeWeight<T>{nullptr, nullptr}, p->chi, p->N, p->n1, spec, fs, AffineView<T>{}};
     PD_TRY(launch_rows<T>(p, pro, st));
     PD_TRY(col_pass<T>(p, 0, 3, false, st));

@@ -197,15 +197,12 @@ extern "C" pd_status pd_solve_mirror(pd_plan *p, double *u, const double *b, con
         }
     }
     // vectors (d x N doubles): the plan's solver vectors, its residual and
-    // weight-field buffers, and for t one run of FP64 spectrum slots from 14 on
-    // (the force passes use slots 0-7 at most); the expanded field lives in u
+    // weight-field buffers, and for t the FP64 spectrum slots behind those of the
+    // force passes; the expanded field lives in u
     double *x = (double *)p->cg_e, *r = (double *)p->cg_r, *pp = (double *)p->cg_p, *v = (double *)p->cg_q;
     double *rh = p->r64, *sv = (double *)p->Gw;
-    double *tv = (double *)p->spec64 + (size_t)14 * p->N;
-    if (p->spec64_slots < 14 + p->dim) {
-        set_error("pd_solve_mirror: plan has too few FP64 spectrum slots");
-        return PD_ERR_ARG;
-    }
+    double *tv = (double *)p->spec64 + (size_t)force_slots_of(p->dim) * p->N;
+    PD_TRY(check_slots<double>(p, force_slots_of(p->dim) + p->dim));
     // r0 = chi_O (L(h) + b), h = 2 (1 - chi_O) g on Gamma
     k_mir_expand<<<kMirBlocks, 256, 0, st>>>(nullptr, mirror, p->chi_om, p->chi, g, u, p->dim, p->N);
     PD_LAUNCH_CHECK();

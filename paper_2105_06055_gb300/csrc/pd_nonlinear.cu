@@ -275,6 +275,7 @@ pd_status force_nl_dim(pd_plan *p, const T *u, T *L, cudaStream_t st)
     using K = NL<D>;
     cx<T> *spec = reinterpret_cast<cx<T> *>(spec_buf<T>(p));
     const int64_t fs = p->N / 2;
+    PD_TRY(check_slots<T>(p, K::INV));
     T *coef = reinterpret_cast<T *>(p->aff_coef);
     // body mean of u
     {

@@ -1095,13 +1095,12 @@ static pd_status plan_create_impl(const pd_problem *pr, const uint8_t *chi_B, co
     PD_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork[1], cudaEventDisableTiming));
 
     // spectra and scratch
-    // the 3D nonlinear bond model's last-axis pass reads 12 and writes 21 spectra (out of place)
-    const int slots = (pr->model == PD_NONLIN_BOND && dim == 3) ? 33 : kMaxSpecFields;
+    const int slots = spec_slots_of(dim, p->nonlinear != 0);
     if (!pr->fp64) {
         p->spec32_slots = slots;
         PD_TRY(dalloc(p, &p->spec32, sizeof(float) * (size_t)p->spec32_slots * N));
     }
-    p->spec64_slots = pr->fp64 ? slots : 8;
+    p->spec64_slots = pr->fp64 ? slots : force_slots_of(dim);
     PD_TRY(dalloc(p, &p->spec64, sizeof(double) * (size_t)p->spec64_slots * N));
     {
         const size_t tb = pr->fp64 ? sizeof(double) : sizeof(float);

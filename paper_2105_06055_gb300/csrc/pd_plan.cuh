@@ -13,9 +13,6 @@
 
 namespace pd {
 
-// Packed-spectrum slots of a plan.
-constexpr int kMaxSpecFields = 20;
-
 // One boundary node of the plan's G field (G != 0 only within delta of the
 // body's boundary): the ncomp components in Sym order and the node index.
 template <typename T>
@@ -30,6 +27,18 @@ template <int D>
 constexpr int kNLFwd = 2 * D + D * (D + 1) / 2;
 template <int D>
 constexpr int kNLInv = D + D * D + D * (D + 1) / 2 + D;
+
+// Packed-spectrum slots of a plan in its own precision: what its widest pass
+// touches, all of them in place. The nonlinear model's inverse fields; the
+// linearized ones' adjoint (two vectors and the symmetric products), which holds the
+// energy's fields and, in 3D, the state-based round's five slots.
+constexpr int spec_slots_of(int dim, bool nonlinear)
+{
+    return nonlinear ? (dim == 2 ? kNLInv<2> : kNLInv<3>) : 2 * dim + dim * (dim + 1) / 2;
+}
+// Slots of one force evaluation without W; in FP64 on FP32 plans (the residual)
+// there is nothing else.
+constexpr int force_slots_of(int dim) { return dim == 2 ? 2 : 5; }
 
 // Device-side view of the model used by the per-node and per-mode functors.
 template <typename T>
@@ -376,6 +385,16 @@ pd_status launch_rows(pd_plan *p, const Op &op, cudaStream_t st, unsigned *grid_
 
 template <typename T>
 inline int spec_slots(const pd_plan *p) { return sizeof(T) == 8 ? p->spec64_slots : p->spec32_slots; }
+
+// PD_ERR_ARG unless the plan has the slots below n (every pipeline asks before its first
+// pass writes them).
+template <typename T>
+pd_status check_slots(const pd_plan *p, int n)
+{
+    if (n <= spec_slots<T>(p)) return PD_OK;
+    set_error("a pass over %d spectra on a plan with %d", n, spec_slots<T>(p));
+    return PD_ERR_ARG;
+}
 
 // Geometry of a column pass along x2 (zaxis 0) or x3 (zaxis 1).
 template <typename T>
