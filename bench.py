@@ -632,7 +632,8 @@ def main():
     ap.add_argument("--n", "--grid", dest="n", type=int, default=N_GRID)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--workload", default="static", choices=["static", "batched", "force"])
-    ap.add_argument("--no-autotune", action="store_true", help="static solve: skip the autotuner of the CG's pass layout (the library's default layout)")
+    ap.add_argument("--no-autotune", action="store_true",
+                    help="static solve: skip the autotuner of the CG's pass layout (the library's default layout)")
     ap.add_argument("--plane-mask", type=int, default=None, metavar="M",
                     help="static solve: halves of the CG iteration run as fused x1-x2 plane passes (bit 0 forward, "
                          "bit 1 inverse; 0 = row and column passes; default: the library's)")

@@ -448,7 +448,7 @@ struct DrSpec {
         ProDR<T, D> pro{e, v, F, p->chi, p->red + kRedScal, p->N, p->n1, spec, fs};
         PD_TRY(launch_rows<T>(p, pro, st));
         if (D == 3) PD_TRY(col_pass<T>(p, 0, D, false, st));
-            CombForce<T, D, false> cmb{m};
+        CombForce<T, D, false> cmb{m};
         PD_TRY(launch_comb<T>(p, cmb, st));
         if (D == 3) PD_TRY(col_pass<T>(p, 0, D, true, st));
         EpiDR<T, D> epi{e, v, rhs, F, p->mbits, m.gent, p->goff, p->red, p->N, p->n1, spec, fs};

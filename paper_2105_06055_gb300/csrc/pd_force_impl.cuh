@@ -14,8 +14,6 @@
 
 namespace pd {
 
-static inline unsigned nblk_f(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
-
 // Fit of the affine split (pd_affine.cuh): block sums over the body, then the
 // exact-form coefficients in the plan's coefficient buffer.
 template <typename T, int D>

@@ -277,12 +277,6 @@ extern "C" pd_status pd_force2d_noalloc(const pd_problem *pr, const uint8_t *chi
     p.spec32_slots = 2;
     p.dev_status = flag + 1;
     p.hdev = hd;
-    {
-        // persistent row-pass grids are sized by the SM count (a query, no allocation)
-        int dev = 0;
-        PD_CUDA_TRY(cudaGetDevice(&dev));
-        PD_CUDA_TRY(cudaDeviceGetAttribute(&p.nsm, cudaDevAttrMultiProcessorCount, dev));
-    }
     const pd_status s = force_bond_pipeline<float, 2, false>(&p, u, nullptr, nullptr, G, L, nullptr, st);
     // the stack plan owns nothing: detach its views before it goes out of scope
     p.chi = nullptr;

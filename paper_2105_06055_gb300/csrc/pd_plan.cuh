@@ -102,11 +102,6 @@ __device__ __forceinline__ void load_ghat_s(const T *t, bool fy, bool fz, T *g)
     g[2] = fz ? -t[2] : t[2];
 }
 
-struct LaunchCfg {
-    dim3 grid, block;
-    size_t smem;
-};
-
 }  // namespace pd
 
 struct pd_plan {
@@ -199,7 +194,8 @@ struct pd_plan {
     double *host_scal = nullptr;    // pinned host copy of the solver scalars
     cudaStream_t own_stream = nullptr;  // plan stream for captured work (never the legacy stream)
     cudaEvent_t ev_join[2] = {nullptr, nullptr};
-    // second stream: the kx = 0 tiles of the 3D last-axis pass run beside the others
+    // second stream: (G p) per boundary entry beside the last-axis pass, for the CG's
+    // inverse plane pass
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t ev_fork[2] = {nullptr, nullptr};
     int no_fork = 0;  // set while capturing into conditional-node bodies (single stream there)

@@ -395,7 +395,7 @@ struct Solver {
         const int64_t fs = p->N / 2;
         const Model<T> m = model_view<T>(p);
         unsigned gpro = 0, gepi = 0;
-            const int lgh = plane_lgh<T, D>(p);
+        const int lgh = plane_lgh<T, D>(p);
         const bool plane_fwd = lgh && (p->plane_passes & 1), plane_inv = lgh && (p->plane_passes & 2);
         const PlaneArgs<T> pa{e, r, pv, q, p->mbits, spec, fs, p->N, p->red, (const T *)p->gpe, p->gnode, p->goff,
                               p->ngent, p->dev_status, p->inject};

@@ -68,7 +68,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, unsigned pha
 }
 
 // The wait after one that ran out, bounded alike. Out of line: inlined it cost the row
-// passes up to 2% in registers and code (128^3 solve 0.6%, so 0.1%).
+// passes up to 2% in registers and code (128^3 solve 0.6 to 2%, so 0.1 to 0.4%).
 static __device__ __noinline__ void mbar_drain(unsigned mbar, unsigned phase)
 {
     const unsigned long long t0 = global_ns();
@@ -117,7 +117,6 @@ __device__ __forceinline__ void bulk_store(void *dst, const void *src, unsigned 
 
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Programmatic dependent launch: wait for the preceding grid of the stream to
 // complete (its memory visible); a no-op when the grid was launched without
 // the programmatic-serialization attribute. The trigger lets the next grid's
@@ -128,7 +127,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // not fill the chip, all blocks of the next pass moved in at once, most of them on
 // the SMs that the pass had left empty, and ran there one after the other. Without
 // it: 64^3 FP64 224 -> 126 us, 1024 x 512 FP32 31 -> 23, 128 x 128 x 64 FP32 41 -> 33,
-// state-based 77 -> 63. Kernels of one block (final reductions) call it.
+// state-based 77 -> 63. Kernels of one block (final reductions) call it, and the body
+// sums (pd_affine.cuh), whose dependent is such a kernel.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // make this thread's generic-proxy shared-memory writes visible to the async proxy
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
